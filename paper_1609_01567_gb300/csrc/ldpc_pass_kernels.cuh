@@ -846,11 +846,14 @@ template <int D, int P, typename M, bool kFirst, bool kSyn, bool kFull, typename
 __device__ __forceinline__ void check_node_pairs_masked(int d, Load &&load, M *out, size_t Fp, const PassArgs &a,
                                                         bool (&unsat)[2 * P]) {
     const float l_max = a.l_max, r_max = a.r_max;
+    // chunk of inputs whose suffix states are held at once (see below)
+    constexpr int C = D <= 8 ? D : 6;
+    constexpr int NC = (D + C - 1) / C;
     float2 tt[D][P];
     // sign bits of the inputs, input k at bit D - 1 - k (shifted in by one
     // funnel shift per input; padding slots shift in 0)
     uint32_t sb[2 * P];
-    uint32_t z[2 * P];
+    uint32_t z[2 * P];  // sign bit: parity of the decisions APP > 0, each the sign of 0 - APP
 #pragma unroll
     for (int v = 0; v < 2 * P; ++v) sb[v] = z[v] = 0u;
 #pragma unroll
@@ -874,8 +877,11 @@ __device__ __forceinline__ void check_node_pairs_masked(int d, Load &&load, M *o
     }
 #pragma unroll
     for (int v = 0; v < 2 * P; ++v) unsat[v] |= z[v] != 0u;
-    // (A2, D) of the inputs after k (the last one's is empty: (2, 0))
-    float2 sa[D][P], sd[D][P];
+    // (A2, D) of the inputs after each chunk (the last one's is empty: (2, 0));
+    // a chunk's own suffix states are formed when its outputs are, the same
+    // merges again, so that wide checks hold C states a frame pair instead of
+    // D (two CTAs per SM instead of one for 18 slots)
+    float2 ea[NC][P], ed[NC][P];
     {
         float2 ca[P], cd[P];
 #pragma unroll
@@ -887,9 +893,11 @@ __device__ __forceinline__ void check_node_pairs_masked(int d, Load &&load, M *o
         for (int k = D - 1; k >= 0; --k) {
 #pragma unroll
             for (int q = 0; q < P; ++q) {
-                sa[k][q] = ca[q];
-                sd[k][q] = cd[q];
-                if (k > 0) pf_merge2(ca[q], cd[q], tt[k][q]);
+                if (k == D - 1 || k % C == C - 1) {
+                    ea[k / C][q] = ca[q];
+                    ed[k / C][q] = cd[q];
+                }
+                if (k >= C) pf_merge2(ca[q], cd[q], tt[k][q]);
             }
         }
     }
@@ -909,28 +917,45 @@ __device__ __forceinline__ void check_node_pairs_masked(int d, Load &&load, M *o
 #pragma unroll
     for (int v = 0; v < 2 * P; ++v) neg[v] = ((dpar ^ __popc(sb[v])) & 1u) ? ~sb[v] : sb[v];
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
-        float2 o[P];
+    for (int ch = 0; ch < NC; ++ch) {
+        float2 sa[C][P], sd[C][P];
 #pragma unroll
         for (int q = 0; q < P; ++q) {
-            // checks of the bin's full degree D >= 4 never need the clamp
-            if (k == 0)
-                o[q] = pf_out_one2<!kFull>(sa[0][q], sd[0][q], r_max);
-            else if (k == D - 1)
-                o[q] = pf_out_one2<!kFull>(pa[q], pd[q], r_max);
-            else
-                o[q] = pf_out2<!kFull>(pa[q], pd[q], sa[k][q], sd[k][q], r_max);
-            o[q].x = with_sign(o[q].x, neg[2 * q] << (32 - D + k));
-            o[q].y = with_sign(o[q].y, neg[2 * q + 1] << (32 - D + k));
-            if (k + 1 < D) pf_merge2(pa[q], pd[q], tt[k][q]);
+            float2 ca = ea[ch][q], cd = ed[ch][q];
+#pragma unroll
+            for (int i = C - 1; i >= 0; --i) {
+                if (ch * C + i >= D) continue;
+                sa[i][q] = ca;
+                sd[i][q] = cd;
+                if (i > 0) pf_merge2(ca, cd, tt[ch * C + i][q]);
+            }
         }
-        if constexpr (kFull && std::is_same_v<M, int8_t> && P == 2) {
-            // |r| <= L <= 20 here (the caller takes this path for int8 only
-            // then), so the levels need no clamp
-            const float x[4] = {o[0].x, o[0].y, o[1].x, o[1].y};
-            MsgIO<int8_t>::store4_unclamped(out + (size_t)k * Fp, x);
-        } else if (kFull || k < d) {
-            store_pairs<M, P>(out + (size_t)k * Fp, o);
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+            const int k = ch * C + i;
+            if (k >= D) continue;
+            float2 o[P];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                // checks of the bin's full degree D >= 4 never need the clamp
+                if (k == 0)
+                    o[q] = pf_out_one2<!kFull>(sa[i][q], sd[i][q], r_max);
+                else if (k == D - 1)
+                    o[q] = pf_out_one2<!kFull>(pa[q], pd[q], r_max);
+                else
+                    o[q] = pf_out2<!kFull>(pa[q], pd[q], sa[i][q], sd[i][q], r_max);
+                o[q].x = with_sign(o[q].x, neg[2 * q] << (32 - D + k));
+                o[q].y = with_sign(o[q].y, neg[2 * q + 1] << (32 - D + k));
+                if (k + 1 < D) pf_merge2(pa[q], pd[q], tt[k][q]);
+            }
+            if constexpr (kFull && std::is_same_v<M, int8_t> && P == 2) {
+                // |r| <= L <= 20 here (the caller takes this path for int8 only
+                // then), so the levels need no clamp
+                const float x[4] = {o[0].x, o[0].y, o[1].x, o[1].y};
+                MsgIO<int8_t>::store4_unclamped(out + (size_t)k * Fp, x);
+            } else if (kFull || k < d) {
+                store_pairs<M, P>(out + (size_t)k * Fp, o);
+            }
         }
     }
 }
@@ -1083,10 +1108,13 @@ struct BulkShape {
 // thread; for 16-bit messages the same bound measured no faster, and wider
 // checks would spill under it). Two for the syndrome form of the other
 // narrow bins, which would otherwise take 136 registers and run one CTA of
-// 8 warps per SM.
+// 8 warps per SM, and for the wider ones wherever two rings fit in shared
+// memory (up to 12 slots, and 16 or 18 slots of 8- and 16-bit messages, which
+// would take 134-161 registers): n = 64800 rate 5/6, int8, 165 frames 2.08 ->
+// 1.88 ms, bfloat16, 256 frames, 10 fixed iterations 1.23 -> 1.11 ms.
 template <int D, typename M, int MODE>
 constexpr int bulk_min_ctas() {
-    return D > 8 ? 1 : (sizeof(M) == 1 ? 3 : (MODE == 2 ? 2 : 1));
+    return D > 8 ? (D <= 12 || sizeof(M) < 4 ? 2 : 1) : (sizeof(M) == 1 ? 3 : (MODE == 2 ? 2 : 1));
 }
 
 template <int D, int V, typename M, int S, int MODE, int RULE>
