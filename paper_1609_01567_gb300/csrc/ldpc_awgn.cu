@@ -8,6 +8,7 @@
 // and permutes the words; the key advances by two Weyl constants per round.
 // Being counter-based, the noise of any (frame, bit) is a pure function of
 // (seed, frame index, bit index), independent of how frames are batched.
+#include <algorithm>
 #include <cmath>
 
 #include "ldpc_internal.h"
@@ -48,37 +49,51 @@ __global__ void k_philox_raw(uint64_t k0, uint64_t k1, uint64_t ctr0, uint64_t c
     }
 }
 
-// One thread per (frame, group of 4 bits).
-__global__ void k_gen_awgn(uint64_t seed, int64_t frame_offset, int32_t F, int32_t n, float sigma, float sigma2,
-                           const uint8_t *__restrict__ cw, float *__restrict__ llr) {
+// One thread per (frame, group of 4 bits): blockIdx.y strides the frames, so no
+// thread divides a 64-bit index by the row length. kVec: rows of whole, aligned
+// groups, read and written four bits at a time. Bound by the integer products
+// of Philox and the logarithm and square root (10,000 frames of 2048 bits 92 ->
+// 83 us); the 128-bit products from four explicit wide products instead of
+// kM * c and __umul64hi ran slower (103 us).
+template <bool kVec>
+__global__ void __launch_bounds__(256) k_gen_awgn(uint64_t seed, int64_t frame_offset, int32_t F, int32_t n, float sigma,
+                                                  float sigma2, const uint8_t *__restrict__ cw,
+                                                  float *__restrict__ llr) {
     const int32_t Q = (n + 3) / 4;
-    const int64_t total = (int64_t)F * Q;
+    const int32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= Q) return;
     const float inv24 = 1.0f / 16777216.0f;
-    for (int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; id < total;
-         id += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t f = (int32_t)(id / Q);
-        const int32_t q = (int32_t)(id - (int64_t)f * Q);
+    for (int32_t f = blockIdx.y; f < F; f += gridDim.y) {
         U64x4 w = philox4x64_10((uint64_t)q, (uint64_t)(frame_offset + f), 0, 0, seed, 0);
         float z[4];
 #pragma unroll
         for (int pair = 0; pair < 2; ++pair) {
-            float ua = (float)((w.x[2 * pair] >> 40) + 1) * inv24;
-            float ub = (float)(w.x[2 * pair + 1] >> 40) * inv24;
+            float ua = (float)(uint32_t)((w.x[2 * pair] >> 40) + 1) * inv24;
+            float ub = (float)(uint32_t)(w.x[2 * pair + 1] >> 40) * inv24;
             float rho = sqrtf(-2.0f * logf(ua));
             float sn, cs;
             sincospif(2.0f * ub, &sn, &cs);
             z[2 * pair] = rho * cs;
             z[2 * pair + 1] = rho * sn;
         }
+        const size_t row = (size_t)f * n + 4 * (size_t)q;
+        float out[4];
+        uint32_t bits = 0;
+        if (kVec && cw) bits = *reinterpret_cast<const uint32_t *>(cw + row);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
-            const int32_t j = 4 * q + t;
-            if (j < n) {
-                const size_t idx = (size_t)f * n + j;
-                float x = cw ? 2.0f * (float)cw[idx] - 1.0f : -1.0f;
-                float y = x + sigma * z[t];
-                llr[idx] = 2.0f * y / sigma2;
-            }
+            uint32_t b = (bits >> (8 * t)) & 0xFFu;
+            if (!kVec && cw && 4 * q + t < n) b = cw[row + t];
+            float x = cw ? 2.0f * (float)b - 1.0f : -1.0f;
+            float y = x + sigma * z[t];
+            out[t] = 2.0f * y / sigma2;
+        }
+        if (kVec) {
+            *reinterpret_cast<float4 *>(llr + row) = make_float4(out[0], out[1], out[2], out[3]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+                if (4 * q + t < n) llr[row + t] = out[t];
         }
     }
 }
@@ -139,12 +154,14 @@ extern "C" int ldpc_gen_awgn(uint64_t seed, int64_t frame_offset, int32_t F, int
     if (frame_offset < 0) return set_error(LDPC_EINVAL, "ldpc_gen_awgn: frame_offset < 0");
     if ((int64_t)F * n == 0) return LDPC_OK;
     if (!llr) return set_error(LDPC_EINVAL, "ldpc_gen_awgn: llr is NULL");
-    const int64_t total = (int64_t)F * ((n + 3) / 4);
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
+    const int32_t Q = (n + 3) / 4;
+    const int32_t threads = Q >= 256 ? 256 : (Q + 31) / 32 * 32;
+    const dim3 grid((unsigned)((Q + threads - 1) / threads), (unsigned)std::min(F, 65535));
     float sigma = (float)std::sqrt((double)sigma2);
-    k_gen_awgn<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(seed, frame_offset, F, n, sigma, sigma2, codewords,
-                                                                    llr);
+    const bool vec = n % 4 == 0 && reinterpret_cast<uintptr_t>(llr) % 16 == 0 &&
+                     reinterpret_cast<uintptr_t>(codewords) % 4 == 0;
+    (vec ? k_gen_awgn<true> : k_gen_awgn<false>)<<<grid, threads, 0, (cudaStream_t)stream>>>(
+        seed, frame_offset, F, n, sigma, sigma2, codewords, llr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "ldpc_gen_awgn: launch");
     return LDPC_OK;
