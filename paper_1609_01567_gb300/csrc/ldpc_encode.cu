@@ -7,17 +7,22 @@
 // Frames travel bit-sliced: word g of a row holds one bit of frames
 // 32g .. 32g + 31, so one XOR combines 32 frames.
 //
-// The dense systematic encoder below serves any code (lifted codes without a
-// staircase included): the host reduces H over GF(2) once, and the device
-// forms each parity bit as the xor of the information bits its reduced row
-// holds.
+// A code whose word fits in shared memory takes one kernel (k_encode_ira). The
+// general path, for longer words and codes with a few very heavy checks:
 //   1. pack      u [F][k] bytes      -> U [k][G] words
 //   2. checks    s_i = xor over the H1 neighbours of check i of U[j], and
 //                its running xor within a chunk of checks
 //   3. carries   exclusive xor-scan of the chunk totals
 //   4. write     c [F][n] bytes: the information bytes, then bit f of
 //                p_i = (running xor) xor (carry of the chunk)
+//
+// The dense systematic encoder serves any code (lifted codes without a
+// staircase included): the host reduces H over GF(2) once, and the device
+// forms each parity bit as the xor of the information bits its reduced row
+// holds.
 #include <algorithm>
+#include <new>
+#include <type_traits>
 #include <vector>
 
 #include "ldpc_internal.h"
@@ -110,37 +115,334 @@ __global__ void k_write_codeword(const uint8_t *__restrict__ info, const uint32_
     }
 }
 
-// Dense systematic encoder (any code): parity row i of the reduced H sets the
-// bit of its pivot column to the xor of the information bits it holds.
-// Bit-sliced like the IRA encoder: P [r][G] from U [k][G].
-__global__ void k_dense_parity(const uint32_t *__restrict__ R, int32_t r, int32_t kw, const uint32_t *__restrict__ U,
-                               int32_t G, uint32_t *__restrict__ P) {
-    const int64_t total = (int64_t)r * G;
-    for (int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; id < total;
-         id += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t i = (int32_t)(id / G);
-        const int32_t g = (int32_t)(id - (int64_t)i * G);
-        const uint32_t *row = R + (size_t)i * kw;
-        uint32_t acc = 0;
-        for (int32_t w = 0; w < kw; ++w)
-            for (uint32_t bits = row[w]; bits; bits &= bits - 1) acc ^= U[(size_t)(32 * w + __ffs(bits) - 1) * G + g];
-        P[(size_t)i * G + g] = acc;
+// ---------------------------------------------------------------------------
+// IRA codes whose word fits in shared memory: one kernel, one CTA per eight
+// frames. A byte of shared memory holds one bit position of the CTA's eight
+// frames. The information bytes are read once, written to the codeword and
+// packed on the way (byte lane b of (w & 0x01..01) << f over f). Each warp
+// forms s_i of a contiguous range of checks, lane = check, from a table with
+// the lanes' entries next to each other, with a running xor by shuffles; after
+// one barrier for the warps' totals it writes its range as bytes of the eight
+// rows, W bytes a store. Bound by the bytes read and written once and by the
+// latency of the table rows between them: n = 64800, 1024 frames 259 -> 36 us
+// against the four kernels of the general path, whose write kernel divides a
+// 64-bit index for every codeword byte (100 MB at the copy rate: 15 us). Rows
+// read through row_ptr and col_idx instead of the padded table: 54 us, every
+// load of a warp touching six lines.
+// ---------------------------------------------------------------------------
+
+template <int W>
+struct Wide;
+template <>
+struct Wide<1> {
+    using T = uint8_t;
+};
+template <>
+struct Wide<4> {
+    using T = uint32_t;
+};
+template <>
+struct Wide<16> {
+    using T = uint4;
+};
+__device__ __forceinline__ uint32_t ones_of(uint8_t x) { return x & 1u; }
+__device__ __forceinline__ uint32_t ones_of(uint32_t x) { return x & 0x01010101u; }
+__device__ __forceinline__ uint4 ones_of(uint4 x) {
+    return make_uint4(x.x & 0x01010101u, x.y & 0x01010101u, x.z & 0x01010101u, x.w & 0x01010101u);
+}
+__device__ __forceinline__ void add_frame(uint32_t &acc, uint32_t x, int f) { acc |= x << f; }
+__device__ __forceinline__ void add_frame(uint4 &acc, uint4 x, int f) {
+    acc.x |= x.x << f;
+    acc.y |= x.y << f;
+    acc.z |= x.z << f;
+    acc.w |= x.w << f;
+}
+__device__ __forceinline__ uint32_t frame_of(uint32_t x, int f) { return (x >> f) & 0x01010101u; }
+__device__ __forceinline__ uint4 frame_of(uint4 x, int f) {
+    return make_uint4(frame_of(x.x, f), frame_of(x.y, f), frame_of(x.z, f), frame_of(x.w, f));
+}
+__device__ __forceinline__ uint32_t flip(uint32_t x, uint32_t c) { return x ^ c; }
+__device__ __forceinline__ uint4 flip(uint4 x, uint32_t c) { return make_uint4(x.x ^ c, x.y ^ c, x.z ^ c, x.w ^ c); }
+
+constexpr int kWordFrames = 8;
+
+// WI: bytes per access of the information part, WP: of the parity part.
+template <int WI, int WP>
+__global__ void __launch_bounds__(1024) k_encode_ira(const uint8_t *__restrict__ info,
+                                                     const int2 *__restrict__ groups,
+                                                     const uint32_t *__restrict__ rows, int32_t F, int32_t m,
+                                                     int32_t k, uint8_t *__restrict__ cw) {
+    extern __shared__ __align__(16) uint8_t es[];
+    uint8_t *U = es;                         // [k] bits of the information positions, then a zero
+    uint8_t *P = es + ((k + 16) & ~15);      // [m] running xor within a warp's range
+    __shared__ uint32_t total[32];
+    const int32_t n = k + m;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
+    const int64_t f0 = (int64_t)blockIdx.x * kWordFrames;
+    const int nf = (int)min((int64_t)kWordFrames, F - f0);
+    {
+        using T = typename Wide<WI>::T;
+        using A = std::conditional_t<WI == 16, uint4, uint32_t>;
+        for (int32_t q = tid; q < k / WI; q += blockDim.x) {
+            A x[kWordFrames];
+#pragma unroll
+            for (int f = 0; f < kWordFrames; ++f)
+                x[f] = f < nf ? ones_of(reinterpret_cast<const T *>(info + (f0 + f) * k)[q]) : A{};
+            A acc{};
+#pragma unroll
+            for (int f = 0; f < kWordFrames; ++f) {
+                add_frame(acc, x[f], f);
+                if (f < nf) {
+                    if constexpr (WI == 1) cw[(f0 + f) * n + q] = (uint8_t)x[f];
+                    else reinterpret_cast<T *>(cw + (f0 + f) * n)[q] = x[f];
+                }
+            }
+            if constexpr (WI == 1) U[q] = (uint8_t)acc;
+            else reinterpret_cast<T *>(U)[q] = acc;
+        }
+    }
+    if (tid == 0) U[k] = 0;
+    __syncthreads();
+    const int32_t per = ((m + warps - 1) / warps + 127) / 128 * 128;
+    const int32_t lo = min(m, warp * per), hi = min(m, lo + per);
+    uint32_t run = 0;
+    for (int32_t i0 = lo; i0 < hi; i0 += 128) {
+        // four groups of 32 checks, byte c of w for group c, so that the shuffles of
+        // the running xor serve four groups
+        uint32_t w = 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int32_t g = i0 / 32 + c;
+            if (32 * g >= hi) continue;
+            const int2 gd = groups[g];  // first entry, entries per lane
+            const uint32_t *p = rows + gd.x + lane;
+            uint32_t x = 0;
+            for (int32_t e = 0; e < gd.y; e += 8) {
+                uint32_t j[8];
+#pragma unroll
+                for (int v = 0; v < 8; ++v) j[v] = e + v < gd.y ? __ldg(p + 32 * (e + v)) : (uint32_t)k;
+#pragma unroll
+                for (int v = 0; v < 8; ++v) x ^= U[j[v]];
+            }
+            w |= x << (8 * c);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w ^= y;
+        }
+        uint32_t t = __shfl_sync(0xffffffffu, w, 31);  // the groups' totals, then the xor of those before
+        t ^= t << 8;
+        t ^= t << 16;
+        w ^= (t << 8) ^ (run * 0x01010101u);
+        run ^= t >> 24;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (i0 + 32 * c + lane < hi) P[i0 + 32 * c + lane] = (uint8_t)(w >> (8 * c));
+    }
+    if (lane == 0) total[warp] = run;
+    __syncthreads();
+    // xor of the totals of the warps before this one, in every byte
+    const uint32_t before = lane < warp ? total[lane] : 0u;
+    const uint32_t carry = __reduce_xor_sync(0xffffffffu, before) * 0x01010101u;
+    for (int32_t q = lo / WP + lane; q < (hi + WP - 1) / WP; q += 32) {
+        using T = typename Wide<WP>::T;
+        using A = std::conditional_t<WP == 16, uint4, uint32_t>;
+        const A x = flip(A(reinterpret_cast<const T *>(P)[q]), carry);
+#pragma unroll
+        for (int f = 0; f < kWordFrames; ++f) {
+            if (f >= nf) break;
+            uint8_t *dst = cw + (f0 + f) * n + k;
+            if constexpr (WP == 1) dst[q] = (uint8_t)frame_of(x, f);
+            else reinterpret_cast<T *>(dst)[q] = frame_of(x, f);
+        }
     }
 }
 
-// c[f][j]: information byte (colmap[j] = its index) or the parity bit of row
-// -1 - colmap[j].
-__global__ void k_dense_write(const uint8_t *__restrict__ info, const uint32_t *__restrict__ P,
-                              const int32_t *__restrict__ colmap, int32_t F, int32_t n, int32_t k, int32_t G,
-                              uint8_t *__restrict__ cw) {
-    const int64_t total = (int64_t)F * n;
-    for (int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; id < total;
-         id += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t f = (int32_t)(id / n);
-        const int32_t j = (int32_t)(id - (int64_t)f * n);
-        const int32_t cm = colmap[j];
-        cw[id] = cm >= 0 ? (uint8_t)(info[(size_t)f * k + cm] & 1u)
-                         : (uint8_t)((P[(size_t)(-1 - cm) * G + (f >> 5)] >> (f & 31)) & 1u);
+constexpr int kEncodeSmem = 224 * 1024;
+
+cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uint32_t *rows, int32_t F, int32_t m,
+                              int32_t k, uint8_t *cw, cudaStream_t s) {
+    const size_t smem = (size_t)((k + 16) & ~15) + ((m + 15) & ~15);
+    const int32_t n = k + m;
+    // a width serves a part when every row start and the part's length are multiples of it
+    auto fits = [&](int w, bool par) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(cw) | (uintptr_t)n | (uintptr_t)k |
+                            (par ? (uintptr_t)m : reinterpret_cast<uintptr_t>(info));
+        return a % w == 0;
+    };
+    const int32_t threads = n <= 2048 ? 128 : (n <= 8192 ? 256 : (n <= 16384 ? 512 : 1024));
+    auto go = [&](auto kernel) {
+        cudaError_t e = cudaSuccess;
+        if (smem > 48 * 1024)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncodeSmem);
+        if (e != cudaSuccess) return e;
+        kernel<<<(unsigned)((F + kWordFrames - 1) / kWordFrames), threads, smem, s>>>(info, groups, rows, F, m, k,
+                                                                                      cw);
+        return cudaGetLastError();
+    };
+    auto pick = [&](auto wi) {
+        constexpr int WI = decltype(wi)::value;
+        if (fits(16, true)) return go(k_encode_ira<WI, 16>);
+        if (fits(4, true)) return go(k_encode_ira<WI, 4>);
+        return go(k_encode_ira<WI, 1>);
+    };
+    if (fits(16, false)) return pick(std::integral_constant<int, 16>{});
+    if (fits(4, false)) return pick(std::integral_constant<int, 4>{});
+    return pick(std::integral_constant<int, 1>{});
+}
+
+// ---------------------------------------------------------------------------
+// Dense systematic encoder (any code): parity row i of the reduced H sets the
+// bit of its pivot column to the xor of the information bits it holds, a
+// product over GF(2). Bit-sliced: word g of a row holds 32 frames, Gp words a
+// row (a multiple of 32, one per lane).
+// ---------------------------------------------------------------------------
+
+// U [k][Gp] from info [F][k]; also clears P [r][Gp]. A CTA packs 4 x 32
+// columns of eight words: lane q reads four bytes of each of a word's 32
+// frames (V4, else byte by byte), and the tile leaves as 32-byte runs.
+template <bool V4>
+__global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ info, int32_t F, int32_t k, int32_t Gp,
+                                                    uint32_t *__restrict__ U, uint32_t *__restrict__ P,
+                                                    int64_t p_words) {
+    __shared__ uint32_t tile[128][9];
+    for (int64_t i = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * 256 + threadIdx.x; i < p_words;
+         i += (int64_t)gridDim.x * gridDim.y * 256)
+        P[i] = 0u;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t j = blockIdx.x * 128 + 4 * lane;
+    const int32_t g = blockIdx.y * 8 + warp;
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {  // eight frames: byte i of acc has column j + i
+        uint32_t acc = 0;
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+            const int64_t fr = 32 * (int64_t)g + 8 * b + f;
+            uint32_t x = 0;
+            if (fr < F) {
+                const uint8_t *src = info + fr * k + j;
+                if (V4) {
+                    if (j < k) x = *reinterpret_cast<const uint32_t *>(src);
+                } else {
+                    for (int i = 0; i < 4; ++i)
+                        if (j + i < k) x |= (uint32_t)src[i] << (8 * i);
+                }
+            }
+            acc |= (x & 0x01010101u) << f;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] |= ((acc >> (8 * i)) & 0xFFu) << (8 * b);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tile[4 * lane + i][warp] = w[i];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 128 * 8; i += 256) {
+        const int32_t c = blockIdx.x * 128 + i / 8;
+        if (c < k) U[(size_t)c * Gp + blockIdx.y * 8 + i % 8] = tile[i / 8][i % 8];
+    }
+}
+
+// P ^= R U over GF(2) by tables (the method of four Russians, Arlazarov,
+// Dinic, Kronrod and Faradzhev 1970): for each four information bits a table
+// of the 16 xors of their words, built once per CTA and read by its kRows
+// parity rows, so a row takes one shared-memory word a lane for four bits
+// instead of two xors on average. A warp's lanes are the 32 words of a group,
+// so every table access is one conflict-free row; a CTA takes a slice of the
+// information bits and adds its part to P by atomic xor. Bound by shared-memory
+// rows and the address arithmetic around them: n = 8192 with 4095 dense rows,
+// 1000 frames: the whole call 264 -> 50 us against a thread walking the set
+// bits of a row, one dependent load each; two CTAs an SM instead of four: 63 us.
+constexpr int kDenseRows = 128;
+constexpr int32_t kDenseFrames = 65536;  // frames per round of kernels (bounds the grids and the scratch)
+
+__global__ void __launch_bounds__(256) k_dense_parity(const uint32_t *__restrict__ R, int32_t r, int32_t k, int32_t kw,
+                                                      int32_t slice, const uint32_t *__restrict__ U, int32_t Gp,
+                                                      uint32_t *__restrict__ P) {
+    __shared__ uint32_t tab[2][8][16][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kPer = kDenseRows / 8;  // rows per warp
+    const int32_t row0 = blockIdx.x * kDenseRows + warp * kPer;
+    const int32_t w0 = blockIdx.y * slice, w1 = min(kw, w0 + slice);
+    const uint32_t *Ug = U + blockIdx.z * 32 + lane;
+    uint32_t acc[kPer];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) acc[i] = 0u;
+    const bool mine = lane < kPer && row0 + lane < r;
+    const uint32_t *Rl = R + (size_t)(mine ? row0 + lane : 0) * kw;
+    uint32_t u[4], rw = 0;
+    auto fetch = [&](int32_t w) {  // this warp's four information words, and its rows' 32 coefficients
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int32_t j = 32 * w + 4 * warp + b;
+            u[b] = w < w1 && j < k ? Ug[(size_t)j * Gp] : 0u;
+        }
+        rw = w < w1 && mine ? Rl[w] : 0u;
+    };
+    fetch(w0);
+    for (int32_t w = w0; w < w1; ++w) {
+        uint32_t(*t)[16][32] = tab[(w - w0) & 1];
+        uint32_t x = 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {  // Gray code: one xor per entry
+            const int code = i ^ (i >> 1);
+            if (i) {
+                const int b = (i & 1) ? 0 : ((i & 2) ? 1 : ((i & 4) ? 2 : 3));
+                x ^= u[b];
+            }
+            t[warp][code][lane] = x;
+        }
+        const uint32_t coef = rw;
+        fetch(w + 1);
+        __syncthreads();  // one barrier a step: the tables alternate
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const uint32_t c = __shfl_sync(0xffffffffu, coef, i);
+            uint32_t y = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) y ^= t[q][(c >> (4 * q)) & 15u][lane];
+            acc[i] ^= y;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+        if (row0 + i < r) atomicXor(P + (size_t)(row0 + i) * Gp + blockIdx.z * 32 + lane, acc[i]);
+}
+
+// c[f][j] from the words of its row: information row colmap[j] of U, or parity
+// row -1 - colmap[j] of P. A thread holds four columns of one word (32
+// frames): byte b of the four words makes eight frames' four bytes.
+template <bool V4>
+__global__ void __launch_bounds__(256) k_dense_write(const uint32_t *__restrict__ U, const uint32_t *__restrict__ P,
+                                                     const int32_t *__restrict__ colmap, int32_t F, int32_t n,
+                                                     int32_t Gp, uint8_t *__restrict__ cw) {
+    const int32_t j = (blockIdx.x * 256 + threadIdx.x) * 4;
+    const int32_t g = blockIdx.y;
+    if (j >= n) return;
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int32_t cm = j + i < n ? colmap[j + i] : 0;
+        w[i] = j + i < n ? (cm >= 0 ? U[(size_t)cm * Gp + g] : P[(size_t)(-1 - cm) * Gp + g]) : 0u;
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const uint32_t s = (uint32_t)(b | (4 + b) << 4);
+        const uint32_t x = __byte_perm(__byte_perm(w[0], w[1], s), __byte_perm(w[2], w[3], s), 0x5410u);
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+            const int64_t fr = 32 * (int64_t)g + 8 * b + f;
+            if (fr >= F) return;
+            const uint32_t y = frame_of(x, f);
+            uint8_t *dst = cw + fr * n + j;
+            if (V4) {
+                *reinterpret_cast<uint32_t *>(dst) = y;
+            } else {
+                for (int i = 0; i < 4; ++i)
+                    if (j + i < n) dst[i] = (uint8_t)(y >> (8 * i));
+            }
+        }
     }
 }
 
@@ -151,6 +453,46 @@ unsigned grid_of(int64_t threads, int per_block, int sm_count) {
 }
 
 }  // namespace
+}  // namespace ldpc
+
+namespace ldpc {
+
+// The information columns of the checks in groups of 32, entry e of a group's
+// lane l at first + 32 e + l (k, a zero bit, where a check has fewer). Not made
+// for a code whose padded table would be four times its edges (a few very
+// heavy checks among light ones): the general path serves it.
+cudaError_t encoder_rows_create(ldpc_code *c) {
+    if (c->ira_k < 0 || c->m == 0 || (size_t)c->n + 48 > (size_t)kEncodeSmem) return cudaSuccess;
+    const uint32_t k = (uint32_t)c->ira_k;
+    try {
+        std::vector<int2> groups;
+        std::vector<uint32_t> rows;
+        for (int32_t i0 = 0; i0 < c->m; i0 += 32) {
+            const int32_t i1 = std::min(c->m, i0 + 32);
+            std::vector<std::vector<uint32_t>> in(32);
+            size_t width = 0;
+            for (int32_t i = i0; i < i1; ++i) {
+                for (int32_t e = c->row_ptr[i]; e < c->row_ptr[i + 1]; ++e)
+                    if ((uint32_t)c->col_idx[e] < k) in[i - i0].push_back((uint32_t)c->col_idx[e]);
+                width = std::max(width, in[i - i0].size());
+            }
+            groups.push_back(make_int2((int)rows.size(), (int)width));
+            for (size_t e = 0; e < width; ++e)
+                for (int l = 0; l < 32; ++l) rows.push_back(e < in[l].size() ? in[l][e] : k);
+            if (rows.size() > 4 * (size_t)c->E + 4096) return cudaSuccess;
+        }
+        cudaError_t e = cudaMalloc(&c->ira_groups, sizeof(int2) * groups.size());
+        if (e == cudaSuccess) e = cudaMalloc(&c->ira_rows, sizeof(uint32_t) * std::max<size_t>(rows.size(), 1));
+        if (e == cudaSuccess)
+            e = cudaMemcpy(c->ira_groups, groups.data(), sizeof(int2) * groups.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !rows.empty())
+            e = cudaMemcpy(c->ira_rows, rows.data(), sizeof(uint32_t) * rows.size(), cudaMemcpyHostToDevice);
+        return e;
+    } catch (const std::bad_alloc &) {
+        return cudaErrorMemoryAllocation;
+    }
+}
+
 }  // namespace ldpc
 
 using namespace ldpc;
@@ -169,6 +511,11 @@ extern "C" int ldpc_encode_ira(ldpc_code_t *c, const uint8_t *info, int32_t n_fr
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(c->device);
+    if (c->ira_groups) {
+        const cudaError_t e = launch_encode_ira(info, c->ira_groups, c->ira_rows, n_frames, m, k, codeword, s);
+        if (prev >= 0) cudaSetDevice(prev);
+        return e == cudaSuccess ? LDPC_OK : cuda_error(e, "ldpc_encode_ira");
+    }
     const int32_t G = (n_frames + 31) / 32;
     // stream-ordered scratch: U [k][G], Pl [m][G] and T [chunks][G] words
     const int32_t nC = (m + kChunk - 1) / kChunk;
@@ -261,6 +608,25 @@ int32_t reduce_parity_check(const ldpc_code *c, std::vector<int32_t> &colmap, st
 
 }  // namespace
 
+// The handle's memory pool of ldpc_encode's scratch: kept between calls up to
+// kEncoderPoolBytes (a pool without a threshold gives its memory back to the
+// driver at every synchronisation: a call followed by one took 461 us, 264 of
+// them its kernels), given back with the handle. Allocation and release are
+// ordered by the caller's stream, so calls on several streams and threads have
+// their own scratch.
+constexpr uint64_t kEncoderPoolBytes = uint64_t(64) << 20;
+
+static cudaError_t encoder_pool(int device, cudaMemPool_t *pool) {
+    cudaMemPoolProps p = {};
+    p.allocType = cudaMemAllocationTypePinned;
+    p.location.type = cudaMemLocationTypeDevice;
+    p.location.id = device;
+    cudaError_t e = cudaMemPoolCreate(pool, &p);
+    uint64_t keep = kEncoderPoolBytes;
+    if (e == cudaSuccess) e = cudaMemPoolSetAttribute(*pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    return e;
+}
+
 extern "C" int ldpc_code_build_encoder(ldpc_code_t *c, int32_t *k_out) {
     if (!c) return set_error(LDPC_EINVAL, "ldpc_code_build_encoder: code is NULL");
     if ((int64_t)c->m * c->n > ((int64_t)1 << 26))
@@ -280,6 +646,7 @@ extern "C" int ldpc_code_build_encoder(ldpc_code_t *c, int32_t *k_out) {
             int32_t *dmap = nullptr;
             cudaError_t e = cudaMalloc(&dR, sizeof(uint32_t) * std::max<size_t>(R.size(), 1));
             if (e == cudaSuccess) e = cudaMalloc(&dmap, sizeof(int32_t) * std::max<size_t>(colmap.size(), 1));
+            if (e == cudaSuccess) e = encoder_pool(c->device, &c->enc_pool);
             if (e == cudaSuccess && !R.empty())
                 e = cudaMemcpy(dR, R.data(), sizeof(uint32_t) * R.size(), cudaMemcpyHostToDevice);
             if (e == cudaSuccess && !colmap.empty())
@@ -288,6 +655,8 @@ extern "C" int ldpc_code_build_encoder(ldpc_code_t *c, int32_t *k_out) {
             if (e != cudaSuccess) {
                 cudaFree(dR);
                 cudaFree(dmap);
+                if (c->enc_pool) cudaMemPoolDestroy(c->enc_pool);
+                c->enc_pool = nullptr;
                 return cuda_error(e, "ldpc_code_build_encoder");
             }
             c->enc_R = dR;
@@ -312,22 +681,35 @@ extern "C" int ldpc_encode(ldpc_code_t *c, const uint8_t *info, int32_t n_frames
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(c->device);
-    const int32_t G = (n_frames + 31) / 32;
     const int32_t kw = (k + 31) / 32;
-    uint32_t *U = nullptr;  // stream-ordered scratch: U [k][G], then P [r][G]
-    const size_t words = ((size_t)k + (size_t)r) * G;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&U), sizeof(uint32_t) * std::max<size_t>(words, 1), s);
+    const int32_t most = std::min(n_frames, kDenseFrames);
+    const int32_t Gp = (most + 1023) / 1024 * 32;  // words a row, 32 to a lane group
+    uint32_t *U = nullptr;  // stream-ordered scratch: U [k][Gp], then P [r][Gp]
+    const size_t words = ((size_t)k + (size_t)r) * Gp;
+    cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&U),
+                                            sizeof(uint32_t) * std::max<size_t>(words, 1), c->enc_pool, s);
     if (e == cudaSuccess) {
-        uint32_t *P = U + (size_t)k * G;
-        if (k > 0) {
-            dim3 grid((unsigned)((k + 255) / 256), (unsigned)std::min(G, 65535));
-            k_pack_info<<<grid, 256, 0, s>>>(info, n_frames, k, G, U);
+        uint32_t *P = U + (size_t)k * Gp;
+        // slices of the information bits until the grid covers the SMs four times
+        const int32_t blocks = (r + kDenseRows - 1) / kDenseRows;
+        const int32_t cover = 4 * std::max(c->sm_count, 1), all = std::max(blocks * (Gp / 32), 1);
+        const int32_t want = std::max(1, std::min(kw, (cover + all - 1) / all));
+        const int32_t slice = std::max(1, (kw + want - 1) / want);
+        for (int32_t f0 = 0; f0 < n_frames; f0 += kDenseFrames) {
+            const int32_t F = std::min(kDenseFrames, n_frames - f0);
+            const uint8_t *in = info + (size_t)f0 * k;
+            uint8_t *out = codeword + (size_t)f0 * n;
+            const dim3 pack((unsigned)std::max((k + 127) / 128, 1), (unsigned)(Gp / 8));
+            const bool in4 = k % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 4 == 0;
+            (in4 ? k_dense_pack<true> : k_dense_pack<false>)<<<pack, 256, 0, s>>>(in, F, k, Gp, U, P, (int64_t)r * Gp);
+            if (r > 0 && k > 0) {
+                const dim3 grid((unsigned)blocks, (unsigned)((kw + slice - 1) / slice), (unsigned)(Gp / 32));
+                k_dense_parity<<<grid, 256, 0, s>>>(c->enc_R, r, k, kw, slice, U, Gp, P);
+            }
+            const dim3 wr((unsigned)((n + 1023) / 1024), (unsigned)((F + 31) / 32));
+            const bool out4 = n % 4 == 0 && reinterpret_cast<uintptr_t>(out) % 4 == 0;
+            (out4 ? k_dense_write<true> : k_dense_write<false>)<<<wr, 256, 0, s>>>(U, P, c->enc_colmap, F, n, Gp, out);
         }
-        if (r > 0)
-            k_dense_parity<<<grid_of((int64_t)r * G, 128, c->sm_count), 128, 0, s>>>(c->enc_R, r, std::max(kw, 1), U,
-                                                                                     G, P);
-        k_dense_write<<<grid_of((int64_t)n_frames * n, 256, c->sm_count), 256, 0, s>>>(info, P, c->enc_colmap, n_frames,
-                                                                                       n, k, G, codeword);
         e = cudaGetLastError();
         cudaError_t e2 = cudaFreeAsync(U, s);
         if (e == cudaSuccess) e = e2;

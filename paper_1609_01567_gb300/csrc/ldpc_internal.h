@@ -57,6 +57,7 @@ struct ProfRecord {
 };
 
 void free_workspace(Workspace &w);
+cudaError_t encoder_rows_create(ldpc_code *c);
 
 // A captured decode: the call's shape, options and buffers, and its graph.
 struct GraphKey {
@@ -130,6 +131,9 @@ struct ldpc_code {
     uint64_t graph_tick = 0;
     cudaStream_t capture_stream = nullptr;
     int32_t debug_giveup_cta = -1;  // ldpc_debug_giveup: armed for the next decode, then cleared
+    // information columns of the checks of an IRA code, for ldpc_encode_ira
+    int2 *ira_groups = nullptr;
+    uint32_t *ira_rows = nullptr;
     // systematic encoder of any code (ldpc_code_build_encoder): enc_k
     // information positions (-1: not built), enc_r = rank of H; on the device
     // the parity rows over the information bits, enc_R [enc_r][ceil(enc_k / 32)]
@@ -138,6 +142,7 @@ struct ldpc_code {
     int32_t enc_k = -1, enc_r = 0;
     uint32_t *enc_R = nullptr;
     int32_t *enc_colmap = nullptr;
+    cudaMemPool_t enc_pool = nullptr;  // ldpc_encode's scratch
 };
 
 namespace ldpc {
