@@ -51,6 +51,7 @@ static void free_device_tables(ldpc_code *c) {
     cudaFree(c->d.phi_table);
     cudaFree(c->d.ms_table);
     cudaFree(c->d.wide_vars);
+    resident_plan_free(&c->resident);
     cudaFree(c->ira_groups);
     cudaFree(c->ira_rows);
     c->ira_groups = nullptr;
@@ -237,6 +238,7 @@ extern "C" int ldpc_code_create(int32_t m, int32_t n, int64_t nnz, const int32_t
             (e = upload(&c->d.wide_vars, c->wide_vars)) != cudaSuccess ||
             (e = upload(&c->d.ms_table, std::vector<float2>((size_t)c->max_cdeg + 1, make_float2(1.0f, 0.0f)))) !=
                 cudaSuccess ||
+            (e = resident_plan_create(c, &c->resident)) != cudaSuccess ||
             (e = encoder_rows_create(c)) != cudaSuccess ||
             (e = cudaEventCreateWithFlags(&c->ws.last_use, cudaEventDisableTiming)) != cudaSuccess) {
             int st = cuda_error(e, "ldpc_code_create: device upload");

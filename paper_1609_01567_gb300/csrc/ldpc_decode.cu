@@ -968,6 +968,17 @@ static int decode_graph(ldpc_code *c, const GraphKey &key, int32_t chunk, cudaSt
 
 static int decode_locked(ldpc_code *c, const float *llr, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o,
                          float l_max, uint8_t *bits, int32_t *iters, uint8_t *ok, float *post, cudaStream_t s) {
+    // a frame that fits in one SM's shared memory stays there (no workspace, one
+    // kernel, nothing shared with other calls)
+    if (c->debug_giveup_cta < 0) {
+        const ResidentShape sh = resident_shape(c, F, o);
+        if (sh.threads) {
+            const cudaError_t e = launch_resident(c, sh, llr, F, max_iter, o, l_max, bits, iters, ok, post, s);
+            if (e != cudaSuccess) return cuda_error(e, "ldpc_decode: kernel launch");
+            c->kernels_launched += 1;
+            return LDPC_OK;
+        }
+    }
     int32_t chunk = std::min(F, kMaxChunkFrames);
     int32_t V, Fp;
     frames_layout(chunk, o.frames_per_lane, &V, &Fp);
@@ -1212,6 +1223,7 @@ struct BatchItem {
     ldpc_code *code = nullptr;
     int32_t F = 0;
     ldpc_decode_opts_t opts{};
+    ResidentShape resident;  // threads > 0: the item runs the resident decode
     Workspace ws;
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
@@ -1220,6 +1232,10 @@ struct BatchItem {
 static cudaError_t enqueue_item(BatchItem &it, int32_t max_iter, float l_max, const float *llr, uint8_t *bits,
                                 int32_t *iters, uint8_t *ok, float *post, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(it.code->mu);
+    if (it.resident.threads) {
+        it.code->kernels_launched += 1;
+        return launch_resident(it.code, it.resident, llr, it.F, max_iter, it.opts, l_max, bits, iters, ok, post, s);
+    }
     return with_msg_type(it.opts.msg_dtype, [&](auto tag) {
         using M = typename decltype(tag)::type;
         return run_chunk<M>(it.code, it.ws, llr, it.F, max_iter, it.opts, l_max, bits, iters, ok, post, nullptr, s);
@@ -1290,6 +1306,7 @@ extern "C" int ldpc_batch_create(int32_t n_items, ldpc_code_t *const *codes, con
         it.code = codes[i];
         it.F = n_frames[i];
         it.opts = o;
+        it.resident = resident_shape(it.code, it.F, o);
         it.opts.streams = 1;      // one branch per item; items overlap each other
         it.opts.tile_frames = 0;
         e = cudaStreamCreateWithFlags(&it.stream, cudaStreamNonBlocking);
@@ -1425,7 +1442,21 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
         }
         float best = 1e30f;
         ldpc_decode_opts_t best_opts = it.opts;
+        const ResidentShape shape = it.resident;
+        float resident_ms = 1e30f;
+        it.resident = ResidentShape{};
         const int32_t lanes[4] = {1, 2, 4, 8};
+        auto timed = [&](float *ms) {
+            for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
+                if (rep == 1) e = cudaEventRecord(t0, it.stream);
+                if (e == cudaSuccess)
+                    e = enqueue_item(it, b->max_iter, b->l_max, llr[i], bits, iters, ok, nullptr, it.stream);
+            }
+            if (e == cudaSuccess) e = cudaEventRecord(t1, it.stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(t1);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(ms, t0, t1);
+            return e;
+        };
         for (int li = 0; li < 4 && status == LDPC_OK; ++li) {
             int32_t v = lanes[li];
             int32_t Fp = (it.F + 32 * v - 1) / (32 * v) * (32 * v);
@@ -1440,14 +1471,7 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
                 it.opts.check_schedule = sched;
                 it.opts.streams = nst;
                 float ms = 0.0f;
-                for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
-                    if (rep == 1) e = cudaEventRecord(t0, it.stream);
-                    if (e == cudaSuccess) e = enqueue_item(it, b->max_iter, b->l_max, llr[i], bits, iters, ok, nullptr,
-                                                           it.stream);
-                }
-                if (e == cudaSuccess) e = cudaEventRecord(t1, it.stream);
-                if (e == cudaSuccess) e = cudaEventSynchronize(t1);
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
+                timed(&ms);
                 if (e != cudaSuccess) {
                     status = cuda_error(e, "ldpc_batch_tune: trial");
                     break;
@@ -1459,6 +1483,12 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
             }
         }
         it.opts = best_opts;
+        // the resident decode against the best of the pass kernels' schedules
+        if (shape.threads && status == LDPC_OK) {
+            it.resident = shape;
+            if (timed(&resident_ms) != cudaSuccess) status = cuda_error(e, "ldpc_batch_tune: trial");
+            if (!(resident_ms < best)) it.resident = ResidentShape{};
+        }
         cudaFree(bits);
         cudaFree(ok);
         cudaFree(iters);

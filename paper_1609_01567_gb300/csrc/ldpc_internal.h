@@ -12,6 +12,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "ldpc_pass.h"
+#include "ldpc_resident.h"
 
 namespace ldpc {
 
@@ -118,6 +119,7 @@ struct ldpc_code {
     int device = -1;
     int sm_count = 0;
     ldpc::DeviceTables d;
+    ldpc::ResidentPlan resident;
     ldpc::Workspace ws;
     std::mutex mu;
     std::vector<ldpc::ProfRecord> prof;

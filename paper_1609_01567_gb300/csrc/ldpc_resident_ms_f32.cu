@@ -1,0 +1,4 @@
+// The resident decode's min-sum kernels with check-to-bit messages stored as float.
+#include "ldpc_resident_kernel.cuh"
+
+LDPC_INSTANTIATE_RESIDENT(float, 1)
