@@ -300,9 +300,9 @@ cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uin
 // ---------------------------------------------------------------------------
 
 // U [k][Gp] from info [F][k]; also clears P [r][Gp]. A CTA packs 4 x 32
-// columns of eight words: lane q reads four bytes of each of a word's 32
-// frames (V4, else byte by byte), and the tile leaves as 32-byte runs.
-template <bool V4>
+// columns of eight words: lane q takes four bytes of each of a word's 32
+// frames, from the one or two aligned words that hold them (rows of k bytes
+// start anywhere), and the tile leaves as 32-byte runs.
 __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ info, int32_t F, int32_t k, int32_t Gp,
                                                     uint32_t *__restrict__ U, uint32_t *__restrict__ P,
                                                     int64_t p_words) {
@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t j = blockIdx.x * 128 + 4 * lane;
     const int32_t g = blockIdx.y * 8 + warp;
+    const int need = min(4, k - j);  // columns of this lane; more bytes than that go nowhere
     uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int b = 0; b < 4; ++b) {  // eight frames: byte i of acc has column j + i
@@ -321,14 +322,11 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
         for (int f = 0; f < 8; ++f) {
             const int64_t fr = 32 * (int64_t)g + 8 * b + f;
             uint32_t x = 0;
-            if (fr < F) {
-                const uint8_t *src = info + fr * k + j;
-                if (V4) {
-                    if (j < k) x = *reinterpret_cast<const uint32_t *>(src);
-                } else {
-                    for (int i = 0; i < 4; ++i)
-                        if (j + i < k) x |= (uint32_t)src[i] << (8 * i);
-                }
+            if (fr < F && need > 0) {
+                const uintptr_t at = reinterpret_cast<uintptr_t>(info + fr * k + j);
+                const uint32_t *w32 = reinterpret_cast<const uint32_t *>(at & ~(uintptr_t)3);
+                const int off = (int)(at & 3);
+                x = __funnelshift_r(w32[0], off + need > 4 ? w32[1] : 0u, 8 * off);
             }
             acc |= (x & 0x01010101u) << f;
         }
@@ -348,27 +346,31 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
 // Dinic, Kronrod and Faradzhev 1970): for each four information bits a table
 // of the 16 xors of their words, built once per CTA and read by its kRows
 // parity rows, so a row takes one shared-memory word a lane for four bits
-// instead of two xors on average. A warp's lanes are the 32 words of a group,
-// so every table access is one conflict-free row; a CTA takes a slice of the
+// instead of two xors on average. A half-warp's lanes are the 32 words of a
+// group, two each, so a table access of a warp reads two conflict-free rows of
+// 128 bytes for two parity rows at once; a CTA takes a slice of the
 // information bits and adds its part to P by atomic xor. Bound by shared-memory
 // rows and the address arithmetic around them: n = 8192 with 4095 dense rows,
-// 1000 frames: the whole call 264 -> 50 us against a thread walking the set
-// bits of a row, one dependent load each; two CTAs an SM instead of four: 63 us.
+// 1000 frames: the whole call 264 -> 39 us against a thread walking the set
+// bits of a row, one dependent load each; a parity row a warp access (one word a
+// lane): 50 us, and with two CTAs an SM instead of four: 63 us.
 constexpr int kDenseRows = 128;
 constexpr int32_t kDenseFrames = 65536;  // frames per round of kernels (bounds the grids and the scratch)
 
 __global__ void __launch_bounds__(256) k_dense_parity(const uint32_t *__restrict__ R, int32_t r, int32_t k, int32_t kw,
                                                       int32_t slice, const uint32_t *__restrict__ U, int32_t Gp,
                                                       uint32_t *__restrict__ P) {
-    __shared__ uint32_t tab[2][8][16][32];
+    __shared__ __align__(16) uint32_t tab[2][8][16][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kPer = kDenseRows / 8;  // rows per warp
     const int32_t row0 = blockIdx.x * kDenseRows + warp * kPer;
     const int32_t w0 = blockIdx.y * slice, w1 = min(kw, w0 + slice);
     const uint32_t *Ug = U + blockIdx.z * 32 + lane;
-    uint32_t acc[kPer];
+    const int half = lane >> 4, pair = lane & 15;  // parity row 2 i + half, words 2 pair and 2 pair + 1
+    const unsigned char *tb = reinterpret_cast<const unsigned char *>(tab);
+    uint2 acc[kPer / 2];
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) acc[i] = 0u;
+    for (int i = 0; i < kPer / 2; ++i) acc[i] = make_uint2(0u, 0u);
     const bool mine = lane < kPer && row0 + lane < r;
     const uint32_t *Rl = R + (size_t)(mine ? row0 + lane : 0) * kw;
     uint32_t u[4], rw = 0;
@@ -396,18 +398,30 @@ __global__ void __launch_bounds__(256) k_dense_parity(const uint32_t *__restrict
         const uint32_t coef = rw;
         fetch(w + 1);
         __syncthreads();  // one barrier a step: the tables alternate
+        const uint32_t at = (uint32_t)pair * 8u + (((w - w0) & 1) ? (uint32_t)sizeof(tab[0]) : 0u);
 #pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const uint32_t c = __shfl_sync(0xffffffffu, coef, i);
-            uint32_t y = 0;
+        for (int i = 0; i < kPer / 2; ++i) {
+            const uint32_t c = __shfl_sync(0xffffffffu, coef, 2 * i + half);
+            uint2 y = make_uint2(0u, 0u);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) y ^= t[q][(c >> (4 * q)) & 15u][lane];
-            acc[i] ^= y;
+            for (int q = 0; q < 8; ++q) {  // byte offset of the entry of bits 4 q .. 4 q + 3: 128 times their value
+                const uint32_t e = (q < 2 ? c << (7 - 4 * q) : c >> (4 * q - 7)) & 0x780u;
+                const uint2 x = *reinterpret_cast<const uint2 *>(tb + q * (int)sizeof(tab[0][0]) + (e | at));
+                y.x ^= x.x;
+                y.y ^= x.y;
+            }
+            acc[i].x ^= y.x;
+            acc[i].y ^= y.y;
         }
     }
 #pragma unroll
-    for (int i = 0; i < kPer; ++i)
-        if (row0 + i < r) atomicXor(P + (size_t)(row0 + i) * Gp + blockIdx.z * 32 + lane, acc[i]);
+    for (int i = 0; i < kPer / 2; ++i) {
+        const int32_t row = row0 + 2 * i + half;
+        if (row >= r) continue;
+        uint32_t *dst = P + (size_t)row * Gp + blockIdx.z * 32 + 2 * pair;
+        atomicXor(dst, acc[i].x);
+        atomicXor(dst + 1, acc[i].y);
+    }
 }
 
 // c[f][j] from the words of its row: information row colmap[j] of U, or parity
@@ -700,8 +714,7 @@ extern "C" int ldpc_encode(ldpc_code_t *c, const uint8_t *info, int32_t n_frames
             const uint8_t *in = info + (size_t)f0 * k;
             uint8_t *out = codeword + (size_t)f0 * n;
             const dim3 pack((unsigned)std::max((k + 127) / 128, 1), (unsigned)(Gp / 8));
-            const bool in4 = k % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 4 == 0;
-            (in4 ? k_dense_pack<true> : k_dense_pack<false>)<<<pack, 256, 0, s>>>(in, F, k, Gp, U, P, (int64_t)r * Gp);
+            k_dense_pack<<<pack, 256, 0, s>>>(in, F, k, Gp, U, P, (int64_t)r * Gp);
             if (r > 0 && k > 0) {
                 const dim3 grid((unsigned)blocks, (unsigned)((kw + slice - 1) / slice), (unsigned)(Gp / 32));
                 k_dense_parity<<<grid, 256, 0, s>>>(c->enc_R, r, k, kw, slice, U, Gp, P);
