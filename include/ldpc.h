@@ -248,7 +248,10 @@ int ldpc_code_set_rule_table(ldpc_code_t *code, int32_t n_degrees, const float *
  *   post_llr  optional device [n_frames][n] float posterior LLRs; NULL to skip
  * The code's decode workspace (device scratch sized for the largest batch
  * seen so far) is allocated on first use and reused; calls that share a code
- * are serialised on the device through an event, whatever their streams.
+ * are serialised on the device through an event, whatever their streams. A
+ * code whose frame fits in one SM's shared memory (up to about n = 16000) is
+ * decoded there by one kernel, with the same results and without the
+ * workspace, unless an option fixes the layout or asks for messages or timing.
  * Errors: LDPC_EINVAL (bad sizes, NULL required pointer), LDPC_ENODEV,
  * LDPC_ENOMEM, LDPC_ECUDA.
  */
@@ -316,8 +319,9 @@ int ldpc_batch_run(ldpc_batch_t *batch, const float *const *llr, uint8_t *const 
 
 /* Autotune each item's kernel schedule (frames per lane in {1, 2, 4, 8} with
  * padding at most the item's own frame count, direct or pipelined check
- * kernel, the item's frames on one stream or split over two) by timing
- * decodes of the given device LLRs; keeps the fastest. Synchronous;
+ * kernel, the item's frames on one stream or split over two, or the whole
+ * decode of a frame on one SM) by timing decodes of the given device LLRs;
+ * keeps the fastest. Synchronous;
  * allocates temporary outputs. */
 int ldpc_batch_tune(ldpc_batch_t *batch, const float *const *llr, void *stream);
 
@@ -464,8 +468,10 @@ int ldpc_gen_bits(uint64_t seed, int64_t frame_offset, int32_t n_frames, int32_t
  * p_i = (H1 u)_i xor p_(i-1), the unique codeword of H with that systematic
  * part (the staircase makes H2 invertible). The paper's simulator takes its
  * codewords as given; this keeps random-codeword simulation on the device.
- * Scratch ((k + m + ceil(m / 64)) * ceil(n_frames / 32) words) is stream-ordered
- * (cudaMallocAsync / cudaFreeAsync on `stream`). Asynchronous.
+ * Words of up to about 229,000 bits take one kernel without scratch; longer
+ * ones (and codes with a few very heavy checks) use stream-ordered scratch of
+ * (k + m + ceil(m / 64)) * ceil(n_frames / 32) words (cudaMallocAsync /
+ * cudaFreeAsync on `stream`). Asynchronous.
  * Errors: LDPC_EINVAL when the code is not in IRA form, for n_frames < 0 or
  * NULL buffers; LDPC_ENODEV for a host-only code.
  */
@@ -490,9 +496,11 @@ int ldpc_code_build_encoder(ldpc_code_t *code, int32_t *k_out);
  * uint8, bit 0 of each byte used, k from ldpc_code_build_encoder) to
  * codewords [n_frames][n] (device uint8): information bit t at the t-th
  * information position, each pivot column the xor its row gives, so that
- * H c = 0 for every frame. Stream-ordered scratch ((k + r) * ceil(n_frames /
- * 32) words). Asynchronous. Errors: LDPC_EINVAL without an encoder, for
- * n_frames < 0 or NULL buffers; LDPC_ENODEV for a host-only code.
+ * H c = 0 for every frame. Stream-ordered scratch ((k + r) * 32 words for each
+ * 1024 frames, at most 65,536 frames at a time) from a memory pool of the handle
+ * that keeps up to 64 MB between calls. Asynchronous. Errors: LDPC_EINVAL
+ * without an encoder, for n_frames < 0 or NULL buffers; LDPC_ENODEV for a
+ * host-only code.
  */
 int ldpc_encode(ldpc_code_t *code, const uint8_t *info, int32_t n_frames, uint8_t *codeword, void *stream);
 

@@ -968,12 +968,14 @@ static int decode_graph(ldpc_code *c, const GraphKey &key, int32_t chunk, cudaSt
 
 static int decode_locked(ldpc_code *c, const float *llr, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o,
                          float l_max, uint8_t *bits, int32_t *iters, uint8_t *ok, float *post, cudaStream_t s) {
-    // a frame that fits in one SM's shared memory stays there (no workspace, one
-    // kernel, nothing shared with other calls)
+    // A frame that fits in one SM's shared memory stays there: one kernel, no
+    // workspace. Calls that share a code run one after the other all the same.
     if (c->debug_giveup_cta < 0) {
-        const ResidentShape sh = resident_shape(c, F, o);
+        const ResidentShape sh = resident_shape(c, F, max_iter, o);
         if (sh.threads) {
-            const cudaError_t e = launch_resident(c, sh, llr, F, max_iter, o, l_max, bits, iters, ok, post, s);
+            cudaError_t e = cudaStreamWaitEvent(s, c->ws.last_use, 0);
+            if (e == cudaSuccess) e = launch_resident(c, sh, llr, F, max_iter, o, l_max, bits, iters, ok, post, s);
+            if (e == cudaSuccess) e = cudaEventRecord(c->ws.last_use, s);
             if (e != cudaSuccess) return cuda_error(e, "ldpc_decode: kernel launch");
             c->kernels_launched += 1;
             return LDPC_OK;
@@ -1306,7 +1308,7 @@ extern "C" int ldpc_batch_create(int32_t n_items, ldpc_code_t *const *codes, con
         it.code = codes[i];
         it.F = n_frames[i];
         it.opts = o;
-        it.resident = resident_shape(it.code, it.F, o);
+        it.resident = resident_shape(it.code, it.F, max_iter, o);
         it.opts.streams = 1;      // one branch per item; items overlap each other
         it.opts.tile_frames = 0;
         e = cudaStreamCreateWithFlags(&it.stream, cudaStreamNonBlocking);

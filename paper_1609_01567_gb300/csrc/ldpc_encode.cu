@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
 
 // P ^= R U over GF(2) by tables (the method of four Russians, Arlazarov,
 // Dinic, Kronrod and Faradzhev 1970): for each four information bits a table
-// of the 16 xors of their words, built once per CTA and read by its kRows
+// of the 16 xors of their words, built once per CTA and read by its kDenseRows
 // parity rows, so a row takes one shared-memory word a lane for four bits
 // instead of two xors on average. A half-warp's lanes are the 32 words of a
 // group, two each, so a table access of a warp reads two conflict-free rows of

@@ -157,7 +157,7 @@ void resident_plan_free(ResidentPlan *p) {
     *p = ResidentPlan{};
 }
 
-ResidentShape resident_shape(const ldpc_code *c, int32_t F, const ldpc_decode_opts_t &o) {
+ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o) {
     ResidentShape sh;
     const ResidentPlan &p = c->resident;
     if (!p.ok || F <= 0 || o.frames_per_lane || o.check_schedule || o.tile_frames || o.streams || o.r_out || o.profile ||
@@ -182,10 +182,22 @@ ResidentShape resident_shape(const ldpc_code *c, int32_t F, const ldpc_decode_op
     // frames 1154 / 822, n = 576, 10,000 frames 543 / 522. Early exit stops every
     // frame on its own and is faster here throughout (n = 16200 int8, 1000 frames
     // 2694 / 2376, one frame n = 1008 149 / 17).
+    // `ahead` is that ratio for full waves of CTAs; a last wave that is not full
+    // takes as long.
     const bool narrow = msg_bytes(o.msg_dtype) < 4;
-    if (!o.early_exit && per_sm <= (narrow ? 2 : 1) && F > (int64_t)per_sm * sms &&
-        (narrow || o.check_rule == LDPC_RULE_SUM_PRODUCT))
-        return ResidentShape{};
+    const int64_t cap = (int64_t)per_sm * sms;
+    // A few frames of a long code leave most SMs idle here, while the passes spread
+    // one frame over all of them (n = 16200, 4 frames, 10 iterations 138 / 172 us,
+    // n = 7152, 5 frames, 50 iterations 408 / 439; n = 6376, 11 frames 184 / 166, n
+    // = 16200, 109 frames 750 / 571). So few iterations that a long code's frames
+    // mostly use them all count as fixed.
+    const bool fixed = !o.early_exit || (max_iter <= 12 && p.slots > 32000);
+    if (fixed && F <= 64 && p.slots > 26000) return ResidentShape{};
+    if (fixed && per_sm <= 2 && F > cap) {
+        const double ahead = (narrow ? 0.7 : 0.9) + 0.1 * per_sm +
+                             (o.check_rule == LDPC_RULE_SUM_PRODUCT ? 0.0 : (narrow ? 0.1 : 0.3));
+        if (ahead * (double)F < (double)((F + cap - 1) / cap * cap)) return ResidentShape{};
+    }
     // Warps of a CTA. 64 registers a thread let 32 warps run on an SM (16 where
     // checks of degree above 12 take 128). With many frames to each SM, few warps
     // a CTA and many CTAs: one CTA's barriers are covered by the others (n = 576,

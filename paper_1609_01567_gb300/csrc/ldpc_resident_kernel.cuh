@@ -258,6 +258,26 @@ __host__ __device__ constexpr bool exact_degree(int DC, int d) {
                       : d == 8 || d == 16 || d == 24 || d == 32;
 }
 
+// Calls f(degree, mask-free) with the form that serves groups of largest degree
+// dm, both as compile-time constants.
+template <int DC, int D, typename F>
+__device__ __forceinline__ void with_form(int dm, bool full, F &&f) {
+    if constexpr (D >= 2) {
+        if constexpr (exact_degree(DC, D)) {
+            if (full && dm == D) {
+                f(std::integral_constant<int, D>{}, std::true_type{});
+                return;
+            }
+        }
+        with_form<DC, D - 1>(dm, full, f);
+    } else if (DC == 4 || dm <= 4) {
+        f(std::integral_constant<int, 4>{}, std::false_type{});
+    } else {
+        f(std::integral_constant<int, DC>{}, std::false_type{});
+    }
+}
+
+// The same for one group, without the closure (see kStay).
 template <int DC, int D, int RULE, bool ZN, int NV, typename M>
 __device__ __forceinline__ bool exact_form(const Group<NV, M> &gr, const unsigned char *app, const ResidentArgs &a,
                                            uint32_t &unsat) {
@@ -280,6 +300,11 @@ template <typename M, int DC, int RULE, bool ZN>
 __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const __grid_constant__ ResidentArgs a) {
     constexpr int kRow = resident_row(DC), NV = kRow / 2;
     constexpr bool kAhead = DC <= 12;  // table rows are fetched one group ahead
+    // a warp stays in a degree's code while its groups have that degree (n = 2048,
+    // 6000 frames, 10 iterations 798 -> 759 us, n = 8192, 700 frames 356 -> 341 us);
+    // wider checks are few to a warp and lose by it (n = 1152, degrees 11 and 12,
+    // 119 -> 129 us, n = 2304 142 -> 151 us)
+    constexpr bool kStay = DC <= 8;
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *flag = reinterpret_cast<uint32_t *>(smem);  // [2]: some check is not satisfied
     float *app = reinterpret_cast<float *>(smem + 16);
@@ -316,6 +341,11 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
             }
         }
     };
+    auto take = [&](Group<NV, M> &gr) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) gr.v[k] = cv[k];
+        gr.r = r + (int)(cw & 0xFFFFu) * 32 + lane;
+    };
     auto fetch_var = [&](int g) {
         if (g < a.n_vg) vv = __ldg(a.v4 + g * 32 + lane);
     };
@@ -343,27 +373,37 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
         // check phase: new messages, and the syndrome of the decision after pass t - 1
         uint32_t unsat = 0u;  // sign bit: a check of this lane is not satisfied
         for (int g = warps - 1 - warp; g < a.n_wc; g += warps) wide_check<RULE, M>(a.wide[g], app, r, a, unsat);
-        for (int g = warp; g < a.n_cg; g += warps) {
-            if constexpr (!kAhead) fetch_check(g);
-            Group<NV, M> gr;
-#pragma unroll
-            for (int i = 0; i < NV; ++i) gr.v[i] = cv[i];
-            const int dm = gr.dm = (int)(cw >> 16) & 63;
-            gr.r = r + (int)(cw & 0xFFFFu) * 32 + lane;
-            const bool full = cw & kResidentFull;
-            gr.zero_neg = a.zero_neg_wide == 2 || (ZN && a.zero_neg_wide == 1);
-            if constexpr (kAhead) fetch_check(g + warps);
-            const unsigned char *ab = smem + 16;
-            if (full && exact_form<DC, DC, RULE, ZN, NV, M>(gr, ab, a, unsat)) continue;
-            if (DC <= 4 || dm <= 4)
-                form<4, false, RULE, ZN, NV, M>(gr, ab, a, unsat);
-            else if constexpr (DC == 6)
-                form<6, false, RULE, ZN, NV, M>(gr, ab, a, unsat);
-            else if constexpr (DC > 4) {
-                if (DC == 8 || dm <= 8)
-                    form<8, false, RULE, ZN, NV, M>(gr, ab, a, unsat);
-                else if constexpr (DC > 8)
-                    form<DC, false, RULE, ZN, NV, M>(gr, ab, a, unsat);
+        if constexpr (kStay) {
+            for (int g = warp; g < a.n_cg;) {
+                const uint32_t kind = cw >> 16;  // degree and mask of this group, and of those that follow it here
+                with_form<DC, DC>((int)kind & 63, (cw & kResidentFull) != 0u, [&](auto dc, auto all) {
+                    Group<NV, M> gr;
+                    gr.dm = (int)kind & 63;
+                    gr.zero_neg = false;
+                    do {
+                        take(gr);
+                        g += warps;
+                        fetch_check(g);
+                        form<decltype(dc)::value, decltype(all)::value, RULE, ZN, NV, M>(gr, smem + 16, a, unsat);
+                    } while (g < a.n_cg && cw >> 16 == kind);
+                });
+            }
+        } else {
+            for (int g = warp; g < a.n_cg; g += warps) {
+                if constexpr (!kAhead) fetch_check(g);
+                Group<NV, M> gr;
+                take(gr);
+                gr.dm = (int)(cw >> 16) & 63;
+                gr.zero_neg = a.zero_neg_wide == 2 || (ZN && a.zero_neg_wide == 1);
+                const bool full = cw & kResidentFull;
+                if constexpr (kAhead) fetch_check(g + warps);
+                if (full && exact_form<DC, DC, RULE, ZN, NV, M>(gr, smem + 16, a, unsat)) continue;
+                if (gr.dm <= 4)
+                    form<4, false, RULE, ZN, NV, M>(gr, smem + 16, a, unsat);
+                else if (gr.dm <= 8)
+                    form<8, false, RULE, ZN, NV, M>(gr, smem + 16, a, unsat);
+                else
+                    form<DC, false, RULE, ZN, NV, M>(gr, smem + 16, a, unsat);
             }
         }
         fetch_var(warp);
@@ -387,29 +427,35 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
             const uint32_t j = a.var[v];
             return j != kResidentPad ? __ldg(llr + j) : 0.0f;
         };
-        for (int g = warp; g < a.n_vg; g += warps) {
-            const uint4 e = vv;
-            fetch_var(g + warps);
-            const int v = g * 32 + lane;
-            float acc = lambda(v);
-            add2(acc, e.x, e.y);
-            if (g < a.n_v3) {  // groups are in falling order of degree
-                add2(acc, e.z, e.w);
-                if (g < a.n_v8) {
-                    const uint4 e8 = __ldg(a.v8 + v);
-                    add2(acc, e8.x, e8.y);
-                    add2(acc, e8.z, e8.w);
-                    if (g < a.n_v16) {
-                        const uint4 x = __ldg(a.v16 + 2 * v), y = __ldg(a.v16 + 2 * v + 1);
-                        add2(acc, x.x, x.y);
-                        add2(acc, x.z, x.w);
-                        add2(acc, y.x, y.y);
-                        add2(acc, y.z, y.w);
-                    }
+        int vg = warp;
+        auto sum_edges = [&](auto kc, int end) {  // groups of variables with up to K edges, below `end`
+            constexpr int K = decltype(kc)::value;
+            for (; vg < end; vg += warps) {
+                const uint4 e = vv;
+                fetch_var(vg + warps);
+                const int v = vg * 32 + lane;
+                float acc = lambda(v);
+                add2(acc, e.x, e.y);
+                if constexpr (K > 2) add2(acc, e.z, e.w);
+                if constexpr (K > 4) {
+                    const uint4 x = __ldg(a.v8 + v);
+                    add2(acc, x.x, x.y);
+                    add2(acc, x.z, x.w);
                 }
+                if constexpr (K > 8) {
+                    const uint4 x = __ldg(a.v16 + 2 * v), y = __ldg(a.v16 + 2 * v + 1);
+                    add2(acc, x.x, x.y);
+                    add2(acc, x.z, x.w);
+                    add2(acc, y.x, y.y);
+                    add2(acc, y.z, y.w);
+                }
+                app[v] = acc;
             }
-            app[v] = acc;
-        }
+        };
+        sum_edges(std::integral_constant<int, 16>{}, a.n_v16);  // groups are in falling order of degree
+        sum_edges(std::integral_constant<int, 8>{}, a.n_v8);
+        sum_edges(std::integral_constant<int, 4>{}, a.n_v3);
+        sum_edges(std::integral_constant<int, 2>{}, a.n_vg);
         // variables of degree above kWideVarDegree: eight partial sums (lane u
         // over edges u, u + 8, ...) added to lambda in order
         for (int g = warps - 1 - warp; g < a.n_wv; g += warps) {
