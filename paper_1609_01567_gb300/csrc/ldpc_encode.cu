@@ -350,12 +350,12 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
 // group, two each, so a table access of a warp reads two conflict-free rows of
 // 128 bytes for two parity rows at once; a CTA takes a slice of the
 // information bits and adds its part to P by atomic xor. Bound by shared-memory
-// rows and the address arithmetic around them: n = 8192 with 4095 dense rows,
+// rows and the address arithmetic around them: n = 8192 with 4093 dense rows,
 // 1000 frames: the whole call 264 -> 39 us against a thread walking the set
 // bits of a row, one dependent load each; a parity row a warp access (one word a
 // lane): 50 us, and with two CTAs an SM instead of four: 63 us.
 constexpr int kDenseRows = 128;
-constexpr int32_t kDenseFrames = 65536;  // frames per round of kernels (bounds the grids and the scratch)
+constexpr int32_t kDenseFrames = 65536;  // frames a launch of each kernel (bounds the grids and the scratch)
 
 __global__ void __launch_bounds__(256) k_dense_parity(const uint32_t *__restrict__ R, int32_t r, int32_t k, int32_t kw,
                                                       int32_t slice, const uint32_t *__restrict__ U, int32_t Gp,
