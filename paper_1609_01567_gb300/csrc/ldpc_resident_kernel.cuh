@@ -6,7 +6,7 @@
 // The arithmetic of a node is that of the pass kernels (ldpc_pass_kernels.cuh),
 // operation for operation, so both decodes give the same results bit for bit.
 //
-// What bounds it: instruction issue (about 80% of the slots at n = 1008 and
+// What bounds it: instruction issue (70-80% of the slots at n = 1008 and
 // 2048) and, with one CTA an SM, the latencies between two barriers; HBM sees a
 // frame's LLRs and decisions once. The pass kernels move a frame's messages
 // through HBM or L2 three times a pass, launch at least two kernels a pass up to
