@@ -165,6 +165,7 @@ __device__ __forceinline__ uint32_t flip(uint32_t x, uint32_t c) { return x ^ c;
 __device__ __forceinline__ uint4 flip(uint4 x, uint32_t c) { return make_uint4(x.x ^ c, x.y ^ c, x.z ^ c, x.w ^ c); }
 
 constexpr int kWordFrames = 8;
+constexpr int kWarpTotals = 32 * sizeof(uint32_t);
 
 // WI: bytes per access of the information part, WP: of the parity part.
 template <int WI, int WP>
@@ -173,9 +174,9 @@ __global__ void __launch_bounds__(1024) k_encode_ira(const uint8_t *__restrict__
                                                      const uint32_t *__restrict__ rows, int32_t F, int32_t m,
                                                      int32_t k, uint8_t *__restrict__ cw) {
     extern __shared__ __align__(16) uint8_t es[];
-    uint8_t *U = es;                         // [k] bits of the information positions, then a zero
-    uint8_t *P = es + ((k + 16) & ~15);      // [m] running xor within a warp's range
-    __shared__ uint32_t total[32];
+    uint32_t *total = reinterpret_cast<uint32_t *>(es);  // [32] xor of a warp's range
+    uint8_t *U = es + kWarpTotals;                       // [k] bits of the information positions, then a zero
+    uint8_t *P = U + ((k + 16) & ~15);                   // [m] running xor within a warp's range
     const int32_t n = k + m;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = blockDim.x >> 5;
     const int64_t f0 = (int64_t)blockIdx.x * kWordFrames;
@@ -259,11 +260,11 @@ __global__ void __launch_bounds__(1024) k_encode_ira(const uint8_t *__restrict__
     }
 }
 
-constexpr int kEncodeSmem = 224 * 1024;
+constexpr int kEncodeSmem = 224 * 1024;  // a word's bits; the warps' totals come on top
 
 cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uint32_t *rows, int32_t F, int32_t m,
                               int32_t k, uint8_t *cw, cudaStream_t s) {
-    const size_t smem = (size_t)((k + 16) & ~15) + ((m + 15) & ~15);
+    const size_t smem = kWarpTotals + (size_t)((k + 16) & ~15) + ((m + 15) & ~15);
     const int32_t n = k + m;
     // a width serves a part when every row start and the part's length are multiples of it
     auto fits = [&](int w, bool par) {
@@ -273,9 +274,11 @@ cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uin
     };
     const int32_t threads = n <= 2048 ? 128 : (n <= 8192 ? 256 : (n <= 16384 ? 512 : 1024));
     auto go = [&](auto kernel) {
+        // all of the kernel's shared memory is dynamic, so that `smem` is what the
+        // 48 KB limit of a launch without the opt-in applies to
         cudaError_t e = cudaSuccess;
         if (smem > 48 * 1024)
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncodeSmem);
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncodeSmem + kWarpTotals);
         if (e != cudaSuccess) return e;
         kernel<<<(unsigned)((F + kWordFrames - 1) / kWordFrames), threads, smem, s>>>(info, groups, rows, F, m, k,
                                                                                       cw);
