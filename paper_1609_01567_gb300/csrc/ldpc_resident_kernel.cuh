@@ -34,7 +34,7 @@ struct Group {
     uint32_t v[NV];
     M *r;  // the slot of input 0; input k is 32 k further
     int dm;
-    bool zero_neg;  // degrees above 16: an input of exactly +0 counts as negative
+    bool zero_neg;  // an input of exactly +0 counts as negative (read where D > 16, whatever the group's degree)
     // entry k of the row, held as packed pairs
     __device__ __forceinline__ uint32_t entry(int k) const { return (k & 1) ? v[k / 2] >> 16 : v[k / 2] & 0xFFFFu; }
 };
@@ -394,7 +394,8 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
                 Group<NV, M> gr;
                 take(gr);
                 gr.dm = (int)(cw >> 16) & 63;
-                gr.zero_neg = a.zero_neg_wide == 2 || (ZN && a.zero_neg_wide == 1);
+                // by the group's own degree: the general form of a wide class serves narrow groups too
+                gr.zero_neg = gr.dm > 16 ? a.zero_neg_wide == 2 || (ZN && a.zero_neg_wide == 1) : ZN;
                 const bool full = cw & kResidentFull;
                 if constexpr (kAhead) fetch_check(g + warps);
                 if (full && exact_form<DC, DC, RULE, ZN, NV, M>(gr, smem + 16, a, unsat)) continue;
