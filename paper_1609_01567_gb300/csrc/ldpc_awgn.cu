@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(256) k_gen_awgn(uint64_t seed, int64_t frame_o
     const int32_t q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= Q) return;
     const float inv24 = 1.0f / 16777216.0f;
-    for (int32_t f = blockIdx.y; f < F; f += gridDim.y) {
+    // 64 bits: f passes 2^31 in its last step where F is close to it
+    for (int64_t f = blockIdx.y; f < F; f += gridDim.y) {
         U64x4 w = philox4x64_10((uint64_t)q, (uint64_t)(frame_offset + f), 0, 0, seed, 0);
         float z[4];
 #pragma unroll

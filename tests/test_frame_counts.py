@@ -1,0 +1,27 @@
+"""Calls whose frame count is close to 2^31: every frame is reached, and no
+frame index wraps. Single frames are compared with short calls."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ldpc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1609_01567_gb300 import build
+    build.build()
+    from paper_1609_01567_gb300 import ldpc as mod
+    return mod
+
+
+def test_channel_noise(ldpc):
+    """Rows of one sample (8.6 GB): the frame loop steps by up to 65,535 frames."""
+    frames = 2 ** 31 - 1
+    llr = torch.full((frames, 1), 7.0e30, device="cuda")
+    ldpc.ldpc_gen_awgn(11, 0, frames, 1, 0.5, out=llr)
+    for at, count in ((0, 4096), (65535 * 17 - 100, 200), (2 ** 30 - 50, 100), (frames - 70000, 70000)):
+        want = ldpc.ldpc_gen_awgn(11, at, count, 1, 0.5)
+        assert torch.equal(llr[at:at + count], want), at
+    assert float(llr.max()) < 1.0e30  # every sample was written
