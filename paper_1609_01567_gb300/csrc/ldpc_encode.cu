@@ -712,8 +712,8 @@ extern "C" int ldpc_encode(ldpc_code_t *c, const uint8_t *info, int32_t n_frames
         const int32_t cover = 4 * std::max(c->sm_count, 1), all = std::max(blocks * (Gp / 32), 1);
         const int32_t want = std::max(1, std::min(kw, (cover + all - 1) / all));
         const int32_t slice = std::max(1, (kw + want - 1) / want);
-        for (int32_t f0 = 0; f0 < n_frames; f0 += kDenseFrames) {
-            const int32_t F = std::min(kDenseFrames, n_frames - f0);
+        for (int64_t f0 = 0; f0 < n_frames; f0 += kDenseFrames) {  // 64 bits: the last step may pass 2^31
+            const int32_t F = (int32_t)std::min<int64_t>(kDenseFrames, n_frames - f0);
             const uint8_t *in = info + (size_t)f0 * k;
             uint8_t *out = codeword + (size_t)f0 * n;
             const dim3 pack((unsigned)std::max((k + 127) / 128, 1), (unsigned)(Gp / 8));

@@ -25,3 +25,15 @@ def test_channel_noise(ldpc):
         want = ldpc.ldpc_gen_awgn(11, at, count, 1, 0.5)
         assert torch.equal(llr[at:at + count], want), at
     assert float(llr.max()) < 1.0e30  # every sample was written
+
+
+def test_dense_encoder(ldpc):
+    """One information bit a word (2.1 GB in, 4.3 GB out), encoded in rounds of
+    65,536 frames: the word repeats its bit."""
+    frames = 2 ** 31 - 64
+    h = ldpc.ldpc_code_create(1, 2, [0, 0], [0, 1])
+    info = torch.empty((frames, 1), dtype=torch.uint8, device="cuda").random_(0, 2)
+    words = torch.full((frames, 2), 2, dtype=torch.uint8, device="cuda")
+    ldpc.ldpc_encode(h, info, out=words)
+    for part, bits in zip(words.split(2 ** 28), info.split(2 ** 28)):
+        assert torch.equal(part, bits.expand(-1, 2))
