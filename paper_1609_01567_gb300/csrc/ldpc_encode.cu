@@ -318,6 +318,22 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
     const int32_t g = blockIdx.y * 8 + warp;
     const int need = min(4, k - j);  // columns of this lane; more bytes than that go nowhere
     uint32_t w[4] = {0u, 0u, 0u, 0u};
+    // The words that hold info's first and last byte reach past its ends where
+    // these are unaligned: put together from their bytes inside it. (Byte loads of
+    // all columns at the ends instead: up to 4 us longer.)
+    const uintptr_t lo = reinterpret_cast<uintptr_t>(info), hi = lo + (size_t)F * k;
+    const uintptr_t first = lo & 3 ? lo & ~(uintptr_t)3 : 0, last = hi & 3 ? hi & ~(uintptr_t)3 : 0;
+    uint32_t head = 0, tail = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (first && first + i >= lo && first + i < hi) head |= (uint32_t)*reinterpret_cast<const uint8_t *>(first + i) << (8 * i);
+        if (last && last + i >= lo && last + i < hi) tail |= (uint32_t)*reinterpret_cast<const uint8_t *>(last + i) << (8 * i);
+    }
+    auto word = [&](uintptr_t a) {
+        uint32_t x = a == first ? head : tail;
+        if (a != first && a != last) x = *reinterpret_cast<const uint32_t *>(a);
+        return x;
+    };
 #pragma unroll
     for (int b = 0; b < 4; ++b) {  // eight frames: byte i of acc has column j + i
         uint32_t acc = 0;
@@ -327,9 +343,9 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
             uint32_t x = 0;
             if (fr < F && need > 0) {
                 const uintptr_t at = reinterpret_cast<uintptr_t>(info + fr * k + j);
-                const uint32_t *w32 = reinterpret_cast<const uint32_t *>(at & ~(uintptr_t)3);
+                const uintptr_t w32 = at & ~(uintptr_t)3;
                 const int off = (int)(at & 3);
-                x = __funnelshift_r(w32[0], off + need > 4 ? w32[1] : 0u, 8 * off);
+                x = __funnelshift_r(word(w32), off + need > 4 ? word(w32 + 4) : 0u, 8 * off);
             }
             acc |= (x & 0x01010101u) << f;
         }

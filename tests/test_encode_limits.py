@@ -55,3 +55,22 @@ def test_longest_words(n):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     encode(n, 114656)
+
+
+# information rows of one to nine bits at every byte offset: the words around the
+# first and the last byte belong to the buffers' neighbours and hold other values
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 9])
+def test_dense_encoder_ends_of_the_information(k):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1609_01567_gb300 import ldpc
+    rows, cols = [0] * (k + 1), list(range(k + 1))  # one check over all bits: the last one is the parity
+    h = ldpc.ldpc_code_create(1, k + 1, rows, cols)
+    assert ldpc.ldpc_code_build_encoder(h) == k
+    for frames in (1, 2, 3, 31, 33):
+        for off in range(4):
+            raw = torch.full((off + frames * k + 8,), 255, dtype=torch.uint8, device="cuda")
+            info = raw[off:off + frames * k].view(frames, k)
+            info.random_(0, 2)
+            want = torch.cat([info, info.sum(1, keepdim=True).remainder(2).to(torch.uint8)], 1)
+            assert torch.equal(ldpc.ldpc_encode(h, info), want), (frames, off)
