@@ -37,3 +37,16 @@ def test_dense_encoder(ldpc):
     ldpc.ldpc_encode(h, info, out=words)
     for part, bits in zip(words.split(2 ** 28), info.split(2 ** 28)):
         assert torch.equal(part, bits.expand(-1, 2))
+
+
+@pytest.mark.parametrize("n", [1, 4, 7, 33, 128, 129, 516, 1023, 1028, 2052])
+def test_channel_noise_of_short_and_odd_rows(ldpc, n):
+    """Frames beside each other in a CTA: every frame's noise is that of the frame
+    alone, and its codeword enters it."""
+    for frames in (1, 2, 700):
+        cw = torch.randint(0, 2, (frames, n), dtype=torch.uint8, device="cuda")
+        for words in (None, cw):
+            llr = ldpc.ldpc_gen_awgn(5, 100, frames, n, 0.8, words)
+            for f in sorted({0, frames // 2, frames - 1}):
+                one = ldpc.ldpc_gen_awgn(5, 100 + f, 1, n, 0.8, None if words is None else words[f:f + 1].clone())
+                assert torch.equal(llr[f:f + 1], one), (frames, f)
