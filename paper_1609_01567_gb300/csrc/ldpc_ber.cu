@@ -2,6 +2,7 @@
 // decoded words and the transmitted ones (or the all-zero word, which is
 // enough by linearity), accumulated on the device.
 #include <algorithm>
+#include <type_traits>
 
 #include "ldpc_internal.h"
 
@@ -71,14 +72,14 @@ __global__ void __launch_bounds__(256) k_count_errors(const uint8_t *__restrict_
     if (threadIdx.x < 4 && sums[threadIdx.x]) atomicAdd(counts + threadIdx.x, sums[threadIdx.x]);
 }
 
-template <int TPF>
+template <int TPF, int W>
 cudaError_t launch_count(const uint8_t *bits, const uint8_t *ref, int32_t F, int32_t n, const int32_t *iters,
                          const uint8_t *ok, unsigned long long *counts, cudaStream_t s) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(bits) | reinterpret_cast<uintptr_t>(ref) | (uintptr_t)n;
-    const unsigned blocks = (unsigned)std::min<int64_t>(((int64_t)F + 256 / TPF - 1) / (256 / TPF), 152 * 4);
-    if (a % 16 == 0) k_count_errors<TPF, 16><<<blocks, 256, 0, s>>>(bits, ref, F, n, iters, ok, counts);
-    else if (a % 4 == 0) k_count_errors<TPF, 4><<<blocks, 256, 0, s>>>(bits, ref, F, n, iters, ok, counts);
-    else k_count_errors<TPF, 1><<<blocks, 256, 0, s>>>(bits, ref, F, n, iters, ok, counts);
+    // byte loads need all the warps an SM holds to keep enough of them in flight
+    // (n = 64801, 1000 frames against a reference: 254 us with four CTAs an SM)
+    const int64_t most = 152 * (W == 1 ? 16 : 4);
+    const unsigned blocks = (unsigned)std::min<int64_t>(((int64_t)F + 256 / TPF - 1) / (256 / TPF), most);
+    k_count_errors<TPF, W><<<blocks, 256, 0, s>>>(bits, ref, F, n, iters, ok, counts);
     return cudaGetLastError();
 }
 
@@ -92,12 +93,20 @@ extern "C" int ldpc_count_errors(const uint8_t *bits, const uint8_t *ref, int32_
     if (!counts) return set_error(LDPC_EINVAL, "ldpc_count_errors: counts is NULL");
     if (n_frames == 0) return LDPC_OK;
     if (n > 0 && !bits) return set_error(LDPC_EINVAL, "ldpc_count_errors: bits is NULL");
-    // a warp per frame, a CTA where a warp alone would walk a long word (more than
-    // eight 16-byte loads a lane)
+    // a warp per frame, a CTA where a warp alone would walk a long word: above 4096
+    // bits (eight 16-byte or 32 four-byte loads a lane; n = 3004, 10,000 frames a warp
+    // 11 us, a CTA 19), byte by byte above 2048 (n = 4095, 1000 frames 16.7 / 12.5 us)
     auto *c = reinterpret_cast<unsigned long long *>(counts);
     const cudaStream_t st = (cudaStream_t)stream;
-    const cudaError_t e = n <= 4096 ? launch_count<32>(bits, ref, n_frames, n, iters, syndrome_ok, c, st)
-                                    : launch_count<256>(bits, ref, n_frames, n, iters, syndrome_ok, c, st);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(bits) | reinterpret_cast<uintptr_t>(ref) | (uintptr_t)n;
+    auto go = [&](auto width) {
+        constexpr int W = decltype(width)::value;
+        return n <= (W == 1 ? 2048 : 4096) ? launch_count<32, W>(bits, ref, n_frames, n, iters, syndrome_ok, c, st)
+                                            : launch_count<256, W>(bits, ref, n_frames, n, iters, syndrome_ok, c, st);
+    };
+    const cudaError_t e = a % 16 == 0  ? go(std::integral_constant<int, 16>{})
+                          : a % 4 == 0 ? go(std::integral_constant<int, 4>{})
+                                       : go(std::integral_constant<int, 1>{});
     if (e != cudaSuccess) return cuda_error(e, "ldpc_count_errors: launch");
     return LDPC_OK;
 }

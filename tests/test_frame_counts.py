@@ -50,3 +50,17 @@ def test_channel_noise_of_short_and_odd_rows(ldpc, n):
             for f in sorted({0, frames // 2, frames - 1}):
                 one = ldpc.ldpc_gen_awgn(5, 100 + f, 1, n, 0.8, None if words is None else words[f:f + 1].clone())
                 assert torch.equal(llr[f:f + 1], one), (frames, f)
+
+
+@pytest.mark.parametrize("n", [2047, 2049, 2052, 4092, 4095, 4098])
+def test_error_counts_of_unaligned_words(ldpc, n):
+    """Loads of one and four bytes on both sides of the lengths where a CTA takes
+    over from a warp, and more frames than CTAs in flight."""
+    for frames in (3, 2500):
+        bits = torch.randint(0, 2, (frames, n), dtype=torch.uint8, device="cuda")
+        ref = torch.randint(0, 2, (frames, n), dtype=torch.uint8, device="cuda")
+        ref[::2] = bits[::2]
+        for r in (None, ref):
+            wrong = (bits != (0 if r is None else r)).sum(1)
+            got = ldpc.ldpc_count_errors(bits, r)
+            assert got.tolist() == [int(wrong.sum()), int((wrong > 0).sum()), 0, 0]
