@@ -974,10 +974,10 @@ static int decode_locked(ldpc_code *c, const float *llr, int32_t F, int32_t max_
         const ResidentShape sh = resident_shape(c, F, max_iter, o);
         if (sh.threads) {
             cudaError_t e = cudaStreamWaitEvent(s, c->ws.last_use, 0);
-            if (e == cudaSuccess) e = launch_resident(c, sh, llr, F, max_iter, o, l_max, bits, iters, ok, post, s);
+            if (e == cudaSuccess)
+                e = launch_resident(c, sh, llr, F, max_iter, o, l_max, bits, iters, ok, post, s, &c->kernels_launched);
             if (e == cudaSuccess) e = cudaEventRecord(c->ws.last_use, s);
             if (e != cudaSuccess) return cuda_error(e, "ldpc_decode: kernel launch");
-            c->kernels_launched += 1;
             return LDPC_OK;
         }
     }
@@ -1234,10 +1234,9 @@ struct BatchItem {
 static cudaError_t enqueue_item(BatchItem &it, int32_t max_iter, float l_max, const float *llr, uint8_t *bits,
                                 int32_t *iters, uint8_t *ok, float *post, cudaStream_t s) {
     std::lock_guard<std::mutex> lock(it.code->mu);
-    if (it.resident.threads) {
-        it.code->kernels_launched += 1;
-        return launch_resident(it.code, it.resident, llr, it.F, max_iter, it.opts, l_max, bits, iters, ok, post, s);
-    }
+    if (it.resident.threads)
+        return launch_resident(it.code, it.resident, llr, it.F, max_iter, it.opts, l_max, bits, iters, ok, post, s,
+                               &it.code->kernels_launched);
     return with_msg_type(it.opts.msg_dtype, [&](auto tag) {
         using M = typename decltype(tag)::type;
         return run_chunk<M>(it.code, it.ws, llr, it.F, max_iter, it.opts, l_max, bits, iters, ok, post, nullptr, s);

@@ -220,7 +220,7 @@ ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, co
 
 cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const float *llr, int32_t F, int32_t max_iter,
                             const ldpc_decode_opts_t &o, float l_max, uint8_t *bits, int32_t *iters, uint8_t *ok,
-                            float *post, cudaStream_t s) {
+                            float *post, cudaStream_t s, int64_t *launched) {
     const ResidentPlan &p = c->resident;
     ResidentArgs a{};
     a.crow = reinterpret_cast<const uint16_t *>(p.tab + p.off[0]);
@@ -260,8 +260,8 @@ cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const f
     a.post = post;
     return with_msg_type(o.msg_dtype, [&](auto tag) {
         using M = typename decltype(tag)::type;
-        return o.check_rule == LDPC_RULE_SUM_PRODUCT ? launch_resident_m<M, 0>(a, p.dclass, sh, s)
-                                                     : launch_resident_m<M, 1>(a, p.dclass, sh, s);
+        return o.check_rule == LDPC_RULE_SUM_PRODUCT ? launch_resident_m<M, 0>(a, p.dclass, sh, s, launched)
+                                                     : launch_resident_m<M, 1>(a, p.dclass, sh, s, launched);
     });
 }
 

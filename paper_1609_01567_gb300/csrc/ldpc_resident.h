@@ -89,11 +89,13 @@ struct ResidentShape {
 };
 ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o);
 
+// Adds the kernels it launches to `launched`.
 cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const float *llr, int32_t F, int32_t max_iter,
                             const ldpc_decode_opts_t &o, float l_max, uint8_t *bits, int32_t *iters, uint8_t *ok,
-                            float *post, cudaStream_t s);
+                            float *post, cudaStream_t s, int64_t *launched);
 
 template <typename M, int RULE>
-cudaError_t launch_resident_m(const ResidentArgs &a, int32_t dclass, const ResidentShape &sh, cudaStream_t s);
+cudaError_t launch_resident_m(const ResidentArgs &a, int32_t dclass, const ResidentShape &sh, cudaStream_t s,
+                              int64_t *launched);
 
 }  // namespace ldpc

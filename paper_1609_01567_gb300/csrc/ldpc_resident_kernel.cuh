@@ -543,16 +543,19 @@ cudaError_t launch_frames(const ResidentArgs &a, int32_t frames, const ResidentS
 }
 
 template <typename M, int DC, int RULE>
-cudaError_t launch(const ResidentArgs &a, const ResidentShape &sh, cudaStream_t s) {
+cudaError_t launch(const ResidentArgs &a, const ResidentShape &sh, cudaStream_t s, int64_t *launched) {
     if constexpr (RULE == 1) {
+        *launched += 1;
         return launch_frames<M, DC, 1, false>(a, a.F, sh, s);
     } else {
         const int32_t plain = std::min(a.F, a.zero_neg_from);
         cudaError_t e = plain > 0 ? launch_frames<M, DC, 0, false>(a, plain, sh, s) : cudaSuccess;
+        *launched += plain > 0 ? 1 : 0;
         if (e == cudaSuccess && plain < a.F) {
             ResidentArgs b = a;
             b.f0 = plain;
             e = launch_frames<M, DC, 0, true>(b, a.F - plain, sh, s);
+            *launched += 1;
         }
         return e;
     }
@@ -561,16 +564,17 @@ cudaError_t launch(const ResidentArgs &a, const ResidentShape &sh, cudaStream_t 
 }  // namespace resident
 
 template <typename M, int RULE>
-cudaError_t launch_resident_m(const ResidentArgs &a, int32_t dclass, const ResidentShape &sh, cudaStream_t s) {
+cudaError_t launch_resident_m(const ResidentArgs &a, int32_t dclass, const ResidentShape &sh, cudaStream_t s,
+                              int64_t *launched) {
     switch (dclass) {
-    case 4: return resident::launch<M, 4, RULE>(a, sh, s);
+    case 4: return resident::launch<M, 4, RULE>(a, sh, s, launched);
     case 6:
-        if constexpr (RULE == 0) return resident::launch<M, 6, RULE>(a, sh, s);
+        if constexpr (RULE == 0) return resident::launch<M, 6, RULE>(a, sh, s, launched);
         [[fallthrough]];
-    case 8: return resident::launch<M, 8, RULE>(a, sh, s);
-    case 12: return resident::launch<M, 12, RULE>(a, sh, s);
-    case 18: return resident::launch<M, 18, RULE>(a, sh, s);
-    default: return resident::launch<M, 32, RULE>(a, sh, s);
+    case 8: return resident::launch<M, 8, RULE>(a, sh, s, launched);
+    case 12: return resident::launch<M, 12, RULE>(a, sh, s, launched);
+    case 18: return resident::launch<M, 18, RULE>(a, sh, s, launched);
+    default: return resident::launch<M, 32, RULE>(a, sh, s, launched);
     }
 }
 
@@ -579,5 +583,5 @@ cudaError_t launch_resident_m(const ResidentArgs &a, int32_t dclass, const Resid
 #define LDPC_INSTANTIATE_RESIDENT(M, RULE)                                                                  \
     namespace ldpc {                                                                                        \
     template cudaError_t launch_resident_m<M, RULE>(const ResidentArgs &, int32_t, const ResidentShape &,   \
-                                                    cudaStream_t);                                          \
+                                                    cudaStream_t, int64_t *);                               \
     }

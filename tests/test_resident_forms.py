@@ -3,6 +3,7 @@ compared bit for bit with the pass kernels (a profiled decode runs those)."""
 import numpy as np
 import pytest
 
+from paper_1609_01567_gb300 import inputs as I
 from tests.test_resident import decodes, ldpc, random_code  # noqa: F401  (ldpc is a fixture)
 
 torch = pytest.importorskip("torch")
@@ -38,3 +39,17 @@ def test_erased_inputs_of_checks_on_both_sides_of_degree_16(ldpc, name, frames):
             got, ref = decodes(ldpc, h, llr, max_iter, early_exit=False, msg_dtype=msg)
             for k in ref:
                 assert torch.equal(got[k], ref[k]), (msg, max_iter, k)
+
+
+def test_kernels_are_counted_as_launched(ldpc):  # noqa: F811
+    """A batch above 8192 frames whose last chunk of passes would hold 1 to 32
+    frames runs as two kernels, other sum-product batches and min-sum as one."""
+    code = I.small_code_n1008()
+    h = ldpc.code_from_inputs(code)
+    llr = torch.full((8200, code.n), -3.0, device="cuda")
+    for frames, rule, kernels in ((8200, "sum_product", 2), (8192, "sum_product", 1), (20, "sum_product", 1),
+                                  (8200, "min_sum", 1)):
+        ldpc.ldpc_prof_read(h, reset=True)
+        ldpc.ldpc_decode(h, llr[:frames], 3, rule=rule, want_post=False)
+        torch.cuda.synchronize()
+        assert ldpc.ldpc_prof_read(h, reset=True)["kernels"] == kernels, (frames, rule)
