@@ -326,7 +326,10 @@ int ldpc_batch_run(ldpc_batch_t *batch, const float *const *llr, uint8_t *const 
 int ldpc_batch_tune(ldpc_batch_t *batch, const float *const *llr, void *stream);
 
 /* The schedule picked for one item (frames per lane, check schedule,
- * streams) and the kernels one graph replay runs. NULL outputs are skipped. */
+ * streams) and the kernels one graph replay runs. streams = 0: the item runs
+ * the decode of a frame on one SM, which has no such schedule; the other two
+ * are then those of its pass kernels, which do not run. NULL outputs are
+ * skipped. */
 int ldpc_batch_info(const ldpc_batch_t *batch, int32_t item, int32_t *frames_per_lane, int32_t *check_schedule,
                     int32_t *streams, int64_t *kernels_per_run);
 

@@ -1507,9 +1507,10 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
 extern "C" int ldpc_batch_info(const ldpc_batch_t *b, int32_t item, int32_t *frames_per_lane, int32_t *check_schedule,
                                int32_t *streams, int64_t *kernels_per_run) {
     if (!b || item < 0 || item >= (int32_t)b->items.size()) return set_error(LDPC_EINVAL, "ldpc_batch_info: bad item");
-    if (frames_per_lane) *frames_per_lane = b->items[item].opts.frames_per_lane;
-    if (check_schedule) *check_schedule = b->items[item].opts.check_schedule;
-    if (streams) *streams = b->items[item].opts.streams;
+    const BatchItem &it = b->items[item];
+    if (frames_per_lane) *frames_per_lane = it.opts.frames_per_lane;
+    if (check_schedule) *check_schedule = it.opts.check_schedule;
+    if (streams) *streams = it.resident.threads ? 0 : it.opts.streams;
     if (kernels_per_run) *kernels_per_run = b->kernels_per_run;
     return LDPC_OK;
 }

@@ -582,6 +582,8 @@ def ldpc_batch_tune(batch: Batch, llrs, stream=None) -> None:
 
 
 def ldpc_batch_info(batch: Batch, item: int) -> dict:
+    """The schedule of one item; ``streams`` 0: it runs the decode of a frame on
+    one SM, and the schedule of its pass kernels is not used."""
     v, s, st, k = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int64()
     _check(library().ldpc_batch_info(batch.handle, item, ctypes.byref(v), ctypes.byref(s), ctypes.byref(st),
                                      ctypes.byref(k)))

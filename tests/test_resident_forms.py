@@ -53,3 +53,20 @@ def test_kernels_are_counted_as_launched(ldpc):  # noqa: F811
         ldpc.ldpc_decode(h, llr[:frames], 3, rule=rule, want_post=False)
         torch.cuda.synchronize()
         assert ldpc.ldpc_prof_read(h, reset=True)["kernels"] == kernels, (frames, rule)
+
+
+def test_batch_info_tells_which_decode_an_item_runs(ldpc):  # noqa: F811
+    """A short code's item runs one kernel (streams 0); with a layout option, or
+    a code too long for one SM, it runs the pass kernels."""
+    short, long_ = I.small_code_n1008(), I.mixed_code(6)
+    hs = [ldpc.code_from_inputs(short), ldpc.code_from_inputs(long_)]
+    assert long_.n == 32400
+    b = ldpc.ldpc_batch_create(hs, [64, 3], 4)
+    assert [ldpc.ldpc_batch_info(b, i)["streams"] for i in range(2)] == [0, 1]
+    llrs = [torch.full((f, h.n), -3.0, device="cuda") for f, h in zip((64, 3), hs)]
+    ldpc.ldpc_prof_read(hs[0], reset=True)
+    ldpc.ldpc_batch_run(b, llrs)
+    torch.cuda.synchronize()
+    assert ldpc.ldpc_prof_read(hs[0], reset=True)["kernels"] == 1
+    b = ldpc.ldpc_batch_create(hs, [64, 3], 4, frames_per_lane=2)
+    assert [ldpc.ldpc_batch_info(b, i)["streams"] for i in range(2)] == [1, 1]
