@@ -1225,7 +1225,8 @@ struct BatchItem {
     ldpc_code *code = nullptr;
     int32_t F = 0;
     ldpc_decode_opts_t opts{};
-    ResidentShape resident;  // threads > 0: the item runs the resident decode
+    ResidentShape fit;       // threads > 0: the item's code and options allow the resident decode
+    ResidentShape resident;  // threads > 0: the item runs it
     Workspace ws;
     cudaStream_t stream = nullptr;
     cudaEvent_t done = nullptr;
@@ -1307,7 +1308,8 @@ extern "C" int ldpc_batch_create(int32_t n_items, ldpc_code_t *const *codes, con
         it.code = codes[i];
         it.F = n_frames[i];
         it.opts = o;
-        it.resident = resident_shape(it.code, it.F, max_iter, o);
+        it.fit = resident_shape(it.code, it.F, max_iter, o);
+        it.resident = it.fit;
         it.opts.streams = 1;      // one branch per item; items overlap each other
         it.opts.tile_frames = 0;
         e = cudaStreamCreateWithFlags(&it.stream, cudaStreamNonBlocking);
@@ -1443,7 +1445,8 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
         }
         float best = 1e30f;
         ldpc_decode_opts_t best_opts = it.opts;
-        const ResidentShape shape = it.resident;
+        const ldpc_decode_opts_t opts_before = it.opts;
+        const ResidentShape resident_before = it.resident;
         float resident_ms = 1e30f;
         it.resident = ResidentShape{};
         const int32_t lanes[4] = {1, 2, 4, 8};
@@ -1485,10 +1488,14 @@ extern "C" int ldpc_batch_tune(ldpc_batch_t *b, const float *const *llr, void *s
         }
         it.opts = best_opts;
         // the resident decode against the best of the pass kernels' schedules
-        if (shape.threads && status == LDPC_OK) {
-            it.resident = shape;
+        if (it.fit.threads && status == LDPC_OK) {
+            it.resident = it.fit;
             if (timed(&resident_ms) != cudaSuccess) status = cuda_error(e, "ldpc_batch_tune: trial");
             if (!(resident_ms < best)) it.resident = ResidentShape{};
+        }
+        if (status != LDPC_OK) {
+            it.opts = opts_before;
+            it.resident = resident_before;
         }
         cudaFree(bits);
         cudaFree(ok);

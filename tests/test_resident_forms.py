@@ -70,3 +70,27 @@ def test_batch_info_tells_which_decode_an_item_runs(ldpc):  # noqa: F811
     assert ldpc.ldpc_prof_read(hs[0], reset=True)["kernels"] == 1
     b = ldpc.ldpc_batch_create(hs, [64, 3], 4, frames_per_lane=2)
     assert [ldpc.ldpc_batch_info(b, i)["streams"] for i in range(2)] == [1, 1]
+
+
+def test_batch_tuning_tries_the_resident_decode_every_time(ldpc):  # noqa: F811
+    """Frames that use all their iterations tune this item to the pass kernels
+    (or nearly); frames that stop early, tuned afterwards, take it back to the
+    resident decode, as in a batch tuned with those alone."""
+    code, entries = I.qc_stand_in_code(16000)
+    h = ldpc.ldpc_code_create_qc(4, 8, 2000, entries)
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    noise = torch.randn((64, code.n), generator=gen, device="cuda")
+    clean = noise - 6.0
+    kw = dict(msg_dtype="bf16")
+    fresh = ldpc.ldpc_batch_create([h], [64], 50, **kw)
+    ldpc.ldpc_batch_tune(fresh, [clean])
+    assert ldpc.ldpc_batch_info(fresh, 0)["streams"] == 0
+    again = ldpc.ldpc_batch_create([h], [64], 50, **kw)
+    ldpc.ldpc_batch_tune(again, [noise])
+    first = ldpc.ldpc_batch_info(again, 0)["streams"]
+    ldpc.ldpc_batch_tune(again, [clean])
+    assert ldpc.ldpc_batch_info(again, 0)["streams"] == 0, first
+    out = ldpc.ldpc_batch_run(again, [clean])[0]
+    ref = ldpc.ldpc_decode(h, clean, 50, profile=True, **kw)
+    for k in ("bits", "iters", "ok"):
+        assert torch.equal(out[k], ref[k]), k
