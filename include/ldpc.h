@@ -248,10 +248,18 @@ int ldpc_code_set_rule_table(ldpc_code_t *code, int32_t n_degrees, const float *
  *   post_llr  optional device [n_frames][n] float posterior LLRs; NULL to skip
  * The code's decode workspace (device scratch sized for the largest batch
  * seen so far) is allocated on first use and reused; calls that share a code
- * are serialised on the device through an event, whatever their streams. A
- * code whose frame fits in one SM's shared memory (up to about n = 16000) is
- * decoded there by one kernel, with the same results and without the
- * workspace, unless an option fixes the layout or asks for messages or timing.
+ * are serialised on the device through an event, whatever their streams.
+ * A code of fewer than 16384 bits (its tables hold 16-bit offsets) whose frame
+ * fits in one SM's 227 KB of shared memory (4 bytes a bit and one message an
+ * edge) may be decoded there by one kernel, with the same results and without
+ * the workspace. That is chosen by an estimate of both decodes' time, and never
+ * with an option that fixes the layout (frames_per_lane, check_schedule,
+ * streams, tile_frames), with profile or r_out (both show the pass kernels, whose times
+ * are then not those of the call without them), or with the tabulated rule.
+ * With early exit it gains most where frames stop early; where most frames use
+ * all their iterations (below the code's threshold), codes above n = 8000 may
+ * take up to 1.45 times the pass kernels' time. A caller that decodes such
+ * frames keeps the pass kernels with streams = 1.
  * Errors: LDPC_EINVAL (bad sizes, NULL required pointer), LDPC_ENODEV,
  * LDPC_ENOMEM, LDPC_ECUDA.
  */

@@ -1308,8 +1308,8 @@ extern "C" int ldpc_batch_create(int32_t n_items, ldpc_code_t *const *codes, con
         it.code = codes[i];
         it.F = n_frames[i];
         it.opts = o;
-        it.fit = resident_shape(it.code, it.F, max_iter, o);
-        it.resident = it.fit;
+        it.fit = resident_shape(it.code, it.F, max_iter, o, true);
+        it.resident = resident_shape(it.code, it.F, max_iter, o);
         it.opts.streams = 1;      // one branch per item; items overlap each other
         it.opts.tile_frames = 0;
         e = cudaStreamCreateWithFlags(&it.stream, cudaStreamNonBlocking);

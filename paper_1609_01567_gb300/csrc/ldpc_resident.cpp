@@ -140,13 +140,14 @@ cudaError_t resident_plan_create(const ldpc_code *c, ResidentPlan *p) {
     }
 }
 
+constexpr int32_t kPassChunk = 8192;  // frames of a chunk of the pass kernels
+
 // The sum-product kernels count an input of exactly +0 as a positive one, all
 // but the register kernel (k_check_reg). The resident decode counts it as the
 // kernel does that serves the check in a decode with passes: frames from
 // `from` on (chunks of up to 32 frames) for degrees up to 16, `wide` above.
 static void zero_sign(const ldpc_code *c, int32_t F, ResidentArgs *a) {
-    constexpr int32_t chunk = 8192;  // frames of a chunk of the pass kernels
-    const int32_t last = F > chunk ? F % chunk : F;
+    const int32_t last = F > kPassChunk ? F % kPassChunk : F;
     a->zero_neg_from = last > 0 && last <= 32 ? F - last : INT_MAX;
     const bool staged = c->bin_off[5] - c->bin_off[4] >= kWideBinAnyKernel;
     a->zero_neg_wide = staged ? 0 : (c->bin_max_degree[4] > 18 ? 2 : 1);  // 2: all frames, 1: from zero_neg_from
@@ -157,7 +158,52 @@ void resident_plan_free(ResidentPlan *p) {
     *p = ResidentPlan{};
 }
 
-ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o) {
+// One iteration of F frames, in us, here and by the pass kernels: estimates for
+// the choice between the two, fitted to 1515 timed pairs of 35 codes of 576 to
+// 16,200 bits (rates 1/3 to 5/6, check degrees 3 to 22 and one of 96, 1 to 5000
+// frames, all message formats, 10 fixed iterations). 9% and 12% root-mean-square off.
+// By the widest check's class: degree 8, 12, 18, 32.
+static int degree_class(const ResidentPlan &p) { return p.dclass <= 8 ? 0 : (p.dclass <= 12 ? 1 : (p.dclass <= 18 ? 2 : 3)); }
+
+// An SM takes a time per message slot (instruction issue) for each of its
+// frames, and latency (barriers) once where several CTAs cover each other's,
+// else for each.
+static double resident_us(const ldpc_code *c, const ResidentShape &sh, int32_t per_sm, int32_t F,
+                          const ldpc_decode_opts_t &o) {
+    constexpr double kSlotNs[2][4] = {{0.249, 0.298, 0.426, 0.485}, {0.235, 0.257, 0.287, 0.352}};
+    constexpr double kLatency = 1.17;
+    const ResidentPlan &p = c->resident;
+    const int32_t sms = std::max(1, c->sm_count), rounds = F / sms + (F % sms != 0);
+    double work = kSlotNs[o.check_rule == LDPC_RULE_SUM_PRODUCT ? 0 : 1][degree_class(p)] * 1e-3 * p.slots;
+    if (!sh.lam_shared) work *= 1.23;
+    if (msg_bytes(o.msg_dtype) == 1) work *= 1.08;
+    return per_sm <= 1 ? rounds * (work + kLatency) : rounds * work + kLatency;
+}
+
+// Launches (one check kernel a degree bin), a time per slot and padded frame,
+// and the messages and posteriors that L2 does not hold at 6.4 TB/s.
+static double passes_us(const ldpc_code *c, int32_t F, const ldpc_decode_opts_t &o) {
+    constexpr double kFramePs[2][4] = {{1.20, 1.96, 2.50, 5.86}, {1.73, 2.12, 2.67, 3.27}};
+    constexpr double kL2 = 47e6;
+    const ResidentPlan &p = c->resident;
+    int bins = 0;
+    for (int b = 0; b < kNumCheckBins; ++b) bins += c->bin_off[b + 1] > c->bin_off[b] ? 1 : 0;
+    const int dc = degree_class(p);
+    const double ps = kFramePs[o.check_rule == LDPC_RULE_SUM_PRODUCT ? 0 : 1][dc];
+    auto chunk = [&](int64_t frames) {
+        // up to 64 frames of narrow checks take the time of 32
+        const double Fp = (double)(frames <= 32 || (frames <= 64 && dc < 3) ? 32 : (frames <= 64 ? 64 : (frames + 127) / 128 * 128));
+        const double bytes = ((double)p.slots * msg_bytes(o.msg_dtype) + 4.0 * c->n) * Fp;
+        return 7.2 + 3.2 * (bins - 1) + 5e-5 * p.slots + ps * 1e-6 * p.slots * Fp +
+               std::max(0.0, bytes - kL2) / 6.4e6;
+    };
+    double us = (F / kPassChunk) * chunk(kPassChunk);
+    if (F % kPassChunk) us += chunk(F % kPassChunk);
+    return us;
+}
+
+ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o,
+                             bool wherever_it_fits) {
     ResidentShape sh;
     const ResidentPlan &p = c->resident;
     if (!p.ok || F <= 0 || o.frames_per_lane || o.check_schedule || o.tile_frames || o.streams || o.r_out || o.profile ||
@@ -172,31 +218,23 @@ ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, co
     if (sh.smem > (size_t)kResidentSmem) return ResidentShape{};
     const int32_t sms = std::max(1, c->sm_count);
     const int32_t per_sm = (int32_t)((size_t)228 * 1024 / (sh.smem + 1024));
-    // Fixed iterations take a frame and pass of the same time either way, and
-    // the pass kernels are the faster ones for long codes in narrow formats,
-    // where only one or two frames fit on an SM and there are more frames than
-    // that: n = 16200 int8, 1000 frames, 10 iterations 821 us against 1072; n =
-    // 8192 int8 717 / 833; n = 10000 bfloat16, 160 frames 225 / 263; FP32, one
-    // frame an SM, 160 frames 249 / 339, 304 frames 353 / 347. Shorter codes and
-    // FP32: n = 4096 bfloat16, 10,000 frames 2459 / 2227, n = 2048 FP32, 6000
-    // frames 1154 / 822, n = 576, 10,000 frames 543 / 522. Early exit stops every
-    // frame on its own and is faster here throughout (n = 16200 int8, 1000 frames
-    // 2694 / 2376, one frame n = 1008 149 / 17).
-    // `ahead` is that ratio for full waves of CTAs; a last wave that is not full
-    // takes as long.
-    const bool narrow = msg_bytes(o.msg_dtype) < 4;
-    const int64_t cap = (int64_t)per_sm * sms;
-    // A few frames of a long code leave most SMs idle here, while the passes spread
-    // one frame over all of them (n = 16200, 4 frames, 10 iterations 138 / 172 us,
-    // n = 7152, 5 frames, 50 iterations 408 / 439; n = 6376, 11 frames 184 / 166, n
-    // = 16200, 109 frames 750 / 571). So few iterations that a long code's frames
-    // mostly use them all count as fixed.
-    const bool fixed = !o.early_exit || (max_iter <= 12 && p.slots > 32000);
-    if (fixed && F <= 64 && p.slots > 26000) return ResidentShape{};
-    if (fixed && per_sm <= 2 && F > cap) {
-        const double ahead = (narrow ? 0.7 : 0.9) + 0.1 * per_sm +
-                             (o.check_rule == LDPC_RULE_SUM_PRODUCT ? 0.0 : (narrow ? 0.1 : 0.3));
-        if (ahead * (double)F < (double)((F + cap - 1) / cap * cap)) return ResidentShape{};
+    // Fixed iterations: the faster one (10 iterations, passes / here: n = 6000 rate
+    // 1/2, 304 frames, half 196 / 147 us; n = 5000 rate 5/6, 1000 frames 1735 / 795;
+    // n = 8000 rate 1/2, int8, 1600 frames 911 / 1079; n = 9000 rate 3/4, 32 frames
+    // 130 / 165). Early exit stops every frame on its own here, while the passes keep
+    // a group of 64-128 frames running until its last one stops and launch up to
+    // max_iter: calls whose frames stop early gain, the more the larger max_iter is
+    // (n = 10000, 620 frames, bfloat16, max_iter 50, 0.4 dB above the code's
+    // threshold 763 / 433 us), and calls whose frames use all their iterations lose an
+    // iteration's ratio (the same 1.5 dB below it 2370 / 2700). A call does not know which it
+    // has, so an iteration may cost up to 1.2 times as much here at max_iter 20 and
+    // 1.4 from 33 on, near where the sums of both losses over the timed codes are
+    // least. streams = 1 keeps the passes. Against the passes, in 35 codes: fixed
+    // iterations at most 1.19 times their time (0.70 in the geometric mean of 2015
+    // calls), frames that never stop 1.45 (0.66 of 2821), that stop 1.17 (0.43 of 6851).
+    if (!wherever_it_fits) {
+        const double limit = o.early_exit ? std::min(1.4, 1.05 + 0.015 * std::max(0, max_iter - 10)) : 1.05;
+        if (resident_us(c, sh, per_sm, F, o) > limit * passes_us(c, F, o)) return ResidentShape{};
     }
     // Warps of a CTA. 64 registers a thread let 32 warps run on an SM (16 where
     // checks of degree above 12 take 128). With many frames to each SM, few warps
@@ -204,15 +242,23 @@ ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, co
     // 3 / 8 warps: 522 / 813 us; n = 1008, 4 / 16 warps 608 / 770 us, 10,000
     // frames, 10 iterations). With few, the slowest frame decides and takes 16
     // warps (n = 1008, 1000 frames, 4 / 8 / 16 warps: 150 / 135 / 133 us; n =
-    // 4096, 355 frames, 8 / 16 warps 433 / 312 us).
+    // 4096, 355 frames, 8 / 16 warps 433 / 312 us), or 32 where no SM has a second
+    // frame (n = 5000, 32 frames, bfloat16, 50 iterations 16 / 32 warps 313 / 255 us).
+    // Short codes of wide checks would leave one CTA an SM by their registers: few
+    // warps there from the second frame of an SM on (n = 576 rate 5/6, 1000 frames, 10
+    // iterations 151 us with nine warps, 70 with four; codes with fewer than
+    // eight frames an SM keep 16: n = 6000 rate 3/4, int8, 400 frames 329 / 486 us).
     const int32_t work = std::max({p.n_cg, (p.n_vg + 1) / 2, 1});  // warps with something to do
     const double per = (double)F / sms;                            // frames to an SM
-    int32_t warps = per_sm <= 1 ? 32 : 16;
+    const int32_t fit = p.dclass <= 12 || o.check_rule != LDPC_RULE_SUM_PRODUCT ? 32 : 16;
+    int32_t warps = per_sm <= 1 || F <= sms ? 32 : 16;
     if (per >= (o.early_exit ? 32 : 8)) {
-        const int32_t fit = p.dclass <= 12 || o.check_rule != LDPC_RULE_SUM_PRODUCT ? 32 : 16;
         warps = std::max((fit + per_sm - 1) / per_sm, std::min(4, p.n_cg));
     } else if (per >= 8 && per_sm >= 4) {
         warps = 8;
+    } else if (fit < 32 && !o.early_exit && per_sm >= 8 && F > sms) {
+        const int32_t at_once = std::min(per_sm, (F + sms - 1) / sms);
+        warps = std::max((fit + at_once - 1) / at_once, std::min(4, p.n_cg));
     }
     sh.threads = 32 * std::min(warps, work);
     return sh;

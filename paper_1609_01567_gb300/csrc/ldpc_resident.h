@@ -81,13 +81,15 @@ cudaError_t resident_plan_create(const ldpc_code *c, ResidentPlan *p);
 void resident_plan_free(ResidentPlan *p);
 
 // Threads and shared memory of a decode of F frames, a CTA each; threads = 0
-// when the resident decode does not serve it.
+// when the resident decode does not serve it, or the pass kernels are the better
+// choice (not asked for wherever_it_fits: a tuner that times both).
 struct ResidentShape {
     int32_t threads = 0;
     bool lam_shared = true;
     size_t smem = 0;
 };
-ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o);
+ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, const ldpc_decode_opts_t &o,
+                             bool wherever_it_fits = false);
 
 // Adds the kernels it launches to `launched`.
 cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const float *llr, int32_t F, int32_t max_iter,

@@ -94,3 +94,26 @@ def test_batch_tuning_tries_the_resident_decode_every_time(ldpc):  # noqa: F811
     ref = ldpc.ldpc_decode(h, clean, 50, profile=True, **kw)
     for k in ("bits", "iters", "ok"):
         assert torch.equal(out[k], ref[k]), k
+
+
+def test_choice_between_one_sm_and_the_passes(ldpc):  # noqa: F811
+    """Few frames of long codes of wide checks, and fixed iterations of many int8
+    frames, run the pass kernels (more than one launch); short codes, and frames
+    that may stop early, run one kernel. Both give the same results."""
+    wide = I.ira_code(16000, 12000, {4: 1.0}, seed=16000)
+    half = I.ira_code(8000, 4000, {6: 1.0}, seed=8000)
+    short = I.small_code_n1008()
+    for code, frames, max_iter, early, msg, one in (
+            (wide, 8, 10, False, "bf16", False), (wide, 8, 50, True, "bf16", False), (half, 1600, 3, False, "i8", False),
+            (half, 1600, 50, True, "i8", True), (half, 100, 10, False, "f16", True), (short, 1, 50, True, "f32", True),
+            (short, 3000, 10, False, "i8", True)):
+        h = ldpc.code_from_inputs(code)
+        gen = torch.Generator(device="cuda").manual_seed(frames)
+        llr = torch.randn((frames, code.n), generator=gen, device="cuda") * 2.0 - 4.0
+        ldpc.ldpc_prof_read(h, reset=True)
+        got = ldpc.ldpc_decode(h, llr, max_iter, early_exit=early, msg_dtype=msg)
+        torch.cuda.synchronize()
+        assert (ldpc.ldpc_prof_read(h, reset=True)["kernels"] == 1) == one, (code.n, frames, max_iter, msg)
+        ref = ldpc.ldpc_decode(h, llr, max_iter, early_exit=early, msg_dtype=msg, streams=1)
+        for k in ref:
+            assert torch.equal(got[k], ref[k]), (code.n, frames, k)
