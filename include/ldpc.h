@@ -480,7 +480,8 @@ int ldpc_gen_bits(uint64_t seed, int64_t frame_offset, int32_t n_frames, int32_t
  * part (the staircase makes H2 invertible). The paper's simulator takes its
  * codewords as given; this keeps random-codeword simulation on the device.
  * Words of up to about 229,000 bits take one kernel without scratch; longer
- * ones (and codes with a few very heavy checks) use stream-ordered scratch of
+ * ones, a few words above about 120,000 bits (fewer than 130 at 200,001), and codes
+ * with a few very heavy checks use stream-ordered scratch of
  * (k + m + ceil(m / 64)) * ceil(n_frames / 32) words (cudaMallocAsync /
  * cudaFreeAsync on `stream`). Asynchronous.
  * Errors: LDPC_EINVAL when the code is not in IRA form, for n_frames < 0 or

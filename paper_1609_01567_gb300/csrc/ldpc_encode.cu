@@ -8,7 +8,8 @@
 // 32g .. 32g + 31, so one XOR combines 32 frames.
 //
 // A code whose word fits in shared memory takes one kernel (k_encode_ira). The
-// general path, for longer words and codes with a few very heavy checks:
+// general path, for longer words, a few long ones and codes with a few very heavy
+// checks:
 //   1. pack      u [F][k] bytes      -> U [k][G] words
 //   2. checks    s_i = xor over the H1 neighbours of check i of U[j], and
 //                its running xor within a chunk of checks
@@ -262,16 +263,29 @@ __global__ void __launch_bounds__(1024) k_encode_ira(const uint8_t *__restrict__
 
 constexpr int kEncodeSmem = 224 * 1024;  // a word's bits; the warps' totals come on top
 
+// Bytes an access of the one-kernel form takes in the information or parity part:
+// every row start and the part's length are multiples of them.
+int ira_width(const uint8_t *info, const uint8_t *cw, int32_t m, int32_t k, bool par) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(cw) | (uintptr_t)(k + m) | (uintptr_t)k |
+                        (par ? (uintptr_t)m : reinterpret_cast<uintptr_t>(info));
+    return a % 16 == 0 ? 16 : (a % 4 == 0 ? 4 : 1);
+}
+
+// Few long words leave most SMs idle in the one-kernel form, whose CTA then takes a
+// time per bit, the more the narrower its accesses are; the general path spreads
+// them over the GPU. n = 200,001, general / one kernel: 8 frames 100 / 146 us, 100
+// frames 142 / 150, 300 frames 244 / 152; n = 130,001, 8 frames 96 / 97; n =
+// 229,000 (four bytes an access) 109 / 119; n = 200,000 (16 bytes) 100 / 86.
+bool ira_one_kernel(int width, int32_t F, int32_t n) {
+    const double ns = width == 16 ? 0.43 : (width == 4 ? 0.52 : 0.53 + 0.0275 * std::min(F, kWordFrames));
+    return ns * 1e-3 * n < 90.0 + 0.45 * F;
+}
+
 cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uint32_t *rows, int32_t F, int32_t m,
                               int32_t k, uint8_t *cw, cudaStream_t s) {
     const size_t smem = kWarpTotals + (size_t)((k + 16) & ~15) + ((m + 15) & ~15);
     const int32_t n = k + m;
-    // a width serves a part when every row start and the part's length are multiples of it
-    auto fits = [&](int w, bool par) {
-        const uintptr_t a = reinterpret_cast<uintptr_t>(cw) | (uintptr_t)n | (uintptr_t)k |
-                            (par ? (uintptr_t)m : reinterpret_cast<uintptr_t>(info));
-        return a % w == 0;
-    };
+    const int wi = ira_width(info, cw, m, k, false), wp = ira_width(info, cw, m, k, true);
     const int32_t threads = n <= 2048 ? 128 : (n <= 8192 ? 256 : (n <= 16384 ? 512 : 1024));
     auto go = [&](auto kernel) {
         // all of the kernel's shared memory is dynamic, so that `smem` is what the
@@ -286,12 +300,12 @@ cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uin
     };
     auto pick = [&](auto wi) {
         constexpr int WI = decltype(wi)::value;
-        if (fits(16, true)) return go(k_encode_ira<WI, 16>);
-        if (fits(4, true)) return go(k_encode_ira<WI, 4>);
+        if (wp == 16) return go(k_encode_ira<WI, 16>);
+        if (wp == 4) return go(k_encode_ira<WI, 4>);
         return go(k_encode_ira<WI, 1>);
     };
-    if (fits(16, false)) return pick(std::integral_constant<int, 16>{});
-    if (fits(4, false)) return pick(std::integral_constant<int, 4>{});
+    if (wi == 16) return pick(std::integral_constant<int, 16>{});
+    if (wi == 4) return pick(std::integral_constant<int, 4>{});
     return pick(std::integral_constant<int, 1>{});
 }
 
@@ -544,7 +558,9 @@ extern "C" int ldpc_encode_ira(ldpc_code_t *c, const uint8_t *info, int32_t n_fr
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(c->device);
-    if (c->ira_groups) {
+    if (c->ira_groups &&
+        ira_one_kernel(std::min(ira_width(info, codeword, m, k, false), ira_width(info, codeword, m, k, true)), n_frames,
+                       n)) {
         const cudaError_t e = launch_encode_ira(info, c->ira_groups, c->ira_rows, n_frames, m, k, codeword, s);
         if (prev >= 0) cudaSetDevice(prev);
         return e == cudaSuccess ? LDPC_OK : cuda_error(e, "ldpc_encode_ira");

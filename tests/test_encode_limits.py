@@ -54,7 +54,8 @@ def test_words_around_48_kilobytes(k, step):
 def test_longest_words(n):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    encode(n, 114656)
+    for frames in (9, 40):  # few words this long take the general path
+        encode(n, 114656, frames)
 
 
 # information rows of one to nine bits at every byte offset: the words around the
@@ -74,3 +75,11 @@ def test_dense_encoder_ends_of_the_information(k):
             info.random_(0, 2)
             want = torch.cat([info, info.sum(1, keepdim=True).remainder(2).to(torch.uint8)], 1)
             assert torch.equal(ldpc.ldpc_encode(h, info), want), (frames, off)
+
+
+# few words of 200,001 bits take the general path, many the one-kernel form
+@pytest.mark.parametrize("frames", [1, 8, 200])
+def test_long_odd_words(frames):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    encode(200001, 100000, frames)
