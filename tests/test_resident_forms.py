@@ -117,3 +117,38 @@ def test_choice_between_one_sm_and_the_passes(ldpc):  # noqa: F811
         ref = ldpc.ldpc_decode(h, llr, max_iter, early_exit=early, msg_dtype=msg, streams=1)
         for k in ref:
             assert torch.equal(got[k], ref[k]), (code.n, frames, k)
+
+
+@pytest.mark.parametrize("rule", ["sum_product", "min_sum"])
+def test_channel_values_outside_shared_memory(ldpc, rule):  # noqa: F811
+    """n = 16200 with FP32 messages: the channel LLRs do not fit beside them."""
+    code = I.mixed_code(5)
+    assert code.n == 16200
+    h = ldpc.code_from_inputs(code)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    llr = torch.randn((304, code.n), generator=gen, device="cuda") * 1.6 - 1.3
+    for early in (True, False):
+        kw = dict(rule=rule, rule_beta=0.15 if rule == "min_sum" else 0.0, early_exit=early)
+        ldpc.ldpc_prof_read(h, reset=True)
+        got = ldpc.ldpc_decode(h, llr, 30 if early else 6, **kw)
+        torch.cuda.synchronize()
+        assert ldpc.ldpc_prof_read(h, reset=True)["kernels"] == 1
+        ref = ldpc.ldpc_decode(h, llr, 30 if early else 6, streams=1, **kw)
+        for k in ref:
+            assert torch.equal(got[k], ref[k]), (early, k)
+
+
+def test_last_chunk_of_few_frames_with_erased_inputs(ldpc):  # noqa: F811
+    """The zero rule changes within a batch above 8192 frames whose last chunk of
+    passes holds 1 to 32."""
+    code = I.small_code_n1008()
+    h = ldpc.code_from_inputs(code)
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    for frames in (8193, 8224, 8225):
+        llr = torch.randn((frames, code.n), generator=gen, device="cuda") * 4.0 - 5.0
+        llr[:, 7::11] = 0.0
+        llr[::5, 3::4] = 0.0
+        got = ldpc.ldpc_decode(h, llr, 6)
+        ref = ldpc.ldpc_decode(h, llr, 6, streams=1)
+        for k in ref:
+            assert torch.equal(got[k], ref[k]), (frames, k)
