@@ -853,7 +853,7 @@ __device__ __forceinline__ void check_node_pairs_masked(int d, Load &&load, M *o
     // sign bits of the inputs, input k at bit D - 1 - k (shifted in by one
     // funnel shift per input; padding slots shift in 0)
     uint32_t sb[2 * P];
-    uint32_t z[2 * P];  // sign bit: parity of the decisions APP > 0, each the sign of 0 - APP
+    uint32_t z[2 * P];  // bit 0: parity of the decisions APP > 0
 #pragma unroll
     for (int v = 0; v < 2 * P; ++v) sb[v] = z[v] = 0u;
 #pragma unroll
