@@ -267,6 +267,7 @@ ResidentShape resident_shape(const ldpc_code *c, int32_t F, int32_t max_iter, co
 cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const float *llr, int32_t F, int32_t max_iter,
                             const ldpc_decode_opts_t &o, float l_max, uint8_t *bits, int32_t *iters, uint8_t *ok,
                             float *post, cudaStream_t s, int64_t *launched) {
+    NvtxRange nvtx_decode("ldpc decode (one SM a frame)");
     const ResidentPlan &p = c->resident;
     ResidentArgs a{};
     a.crow = reinterpret_cast<const uint16_t *>(p.tab + p.off[0]);
