@@ -142,8 +142,8 @@ cudaError_t resident_plan_create(const ldpc_code *c, ResidentPlan *p) {
 
 constexpr int32_t kPassChunk = 8192;  // frames of a chunk of the pass kernels
 
-// The sum-product kernels count an input of exactly +0 as a positive one, all
-// but the register kernel (k_check_reg). The resident decode counts it as the
+// The sum-product kernels count an input of exactly +0, or NaN, as a positive one,
+// all but the register kernel (k_check_reg). The resident decode counts it as the
 // kernel does that serves the check in a decode with passes: frames from
 // `from` on (chunks of up to 32 frames) for degrees up to 16, `wide` above.
 static void zero_sign(const ldpc_code *c, int32_t F, ResidentArgs *a) {

@@ -64,7 +64,7 @@ struct ResidentArgs {
     int32_t n, F, f0, slots;  // frames f0 + blockIdx.x
     int32_t max_iter, early;
     int32_t lam_shared;  // channel LLRs kept in shared memory (else re-read from llr)
-    // an input of exactly +0 counts as negative: frames from zero_neg_from on; in checks of degree above 16
+    // an input of exactly +0, or NaN, counts as negative: frames from zero_neg_from on; in checks of degree above 16
     // never (0), as the others (1) or always (2)
     int32_t zero_neg_from, zero_neg_wide;
     float l_max, phi_lmax, r_max, ms_alpha, ms_beta;

@@ -34,7 +34,7 @@ struct Group {
     uint32_t v[NV];
     M *r;  // the slot of input 0; input k is 32 k further
     int dm;
-    bool zero_neg;  // an input of exactly +0 counts as negative (read where D > 16, whatever the group's degree)
+    bool zero_neg;  // an input of exactly +0, or NaN, counts as negative (read where D > 16, whatever the group's degree)
     // entry k of the row, held as packed pairs
     __device__ __forceinline__ uint32_t entry(int k) const { return (k & 1) ? v[k / 2] >> 16 : v[k / 2] & 0xFFFFu; }
 };
@@ -64,7 +64,8 @@ __device__ __forceinline__ void sp_group(const Group<NV, M> &gr, const unsigned 
         const bool on = kAll || c != kResidentPad;
         const float av = *reinterpret_cast<const float *>(app + (on ? c : 0u));
         float q = extrinsic(av, MsgIO<M>::load1(gr.r + 32 * k));
-        if ((D > 16 ? gr.zero_neg : ZN) && q == 0.0f) q = -0.0f;
+        // what is not above zero, NaN included: the sign of its bit in sb
+        if ((D > 16 ? gr.zero_neg : ZN) && !(q > 0.0f)) q = __uint_as_float(__float_as_uint(q) | 0x80000000u);
         const float e = exp_neg(fminf(fabsf(q), a.l_max));
         z ^= on ? __float_as_uint(__fsub_rn(0.0f, av)) : 0u;
         sb = __funnelshift_l(on ? __float_as_uint(q) : 0u, sb, 1);

@@ -152,3 +152,24 @@ def test_last_chunk_of_few_frames_with_erased_inputs(ldpc):  # noqa: F811
         ref = ldpc.ldpc_decode(h, llr, 6, streams=1)
         for k in ref:
             assert torch.equal(got[k], ref[k]), (frames, k)
+
+
+@pytest.mark.parametrize("frames", [3, 33, 70])
+@pytest.mark.parametrize("degrees", [[3, 4, 6], [7, 12], [5, 17, 18], [8, 25]])
+def test_nan_inputs(ldpc, degrees, frames):  # noqa: F811
+    """A channel value that is no number enters every check as it does in the
+    pass kernels, and spoils the same decisions."""
+    m, n = 97, 410
+    rows, cols = random_code(m, n, degrees, seed=sum(degrees))
+    h = ldpc.ldpc_code_create(m, n, rows, cols)
+    gen = torch.Generator(device="cuda").manual_seed(frames)
+    llr = torch.randn((frames, n), generator=gen, device="cuda") * 4.0 - 3.0
+    llr[::2, 5::37] = float("nan")
+    for msg in ("f32", "f16", "bf16", "i8"):
+        for rule in ("sum_product", "min_sum"):
+            for max_iter in (0, 1, 7):
+                got, ref = decodes(ldpc, h, llr, max_iter, early_exit=False, msg_dtype=msg, rule=rule)
+                for k in ref:
+                    assert torch.equal(torch.nan_to_num(got[k].float(), 123.0), torch.nan_to_num(ref[k].float(), 123.0)), (
+                        msg, rule, max_iter, k)
+                assert torch.equal(got["post"].isnan(), ref["post"].isnan())
