@@ -38,7 +38,8 @@ static cudaError_t make_plan(const ldpc_code *c, ResidentPlan *p) {
     }
     for (int32_t j = 0; j < c->n; ++j)
         (c->col_ptr[j + 1] - c->col_ptr[j] > kWideVarDegree ? wide_vars : vars).push_back(j);
-    const auto vg = degree_groups(vars, c->col_ptr, {});
+    // variables without a check keep their channel value as it is: their own groups
+    const auto vg = degree_groups(vars, c->col_ptr, {0});
     // outputs of checks of up to four inputs can saturate, and the sign of an
     // input of exactly zero changes above 16 (see zero_sign)
     const auto cg = degree_groups(checks, c->row_ptr, {4, 16});
@@ -87,6 +88,7 @@ static cudaError_t make_plan(const ldpc_code *c, ResidentPlan *p) {
     std::vector<uint32_t> v4, v8, v16;
     for (const auto &g : vg) {
         const int32_t d0 = degree(c->col_ptr, g[0]);
+        p->n_v1 += d0 > 0 ? 1 : 0;
         p->n_v3 += d0 > 2 ? 1 : 0;
         p->n_v8 += d0 > 4 ? 1 : 0;
         p->n_v16 += d0 > 8 ? 1 : 0;
@@ -282,6 +284,7 @@ cudaError_t launch_resident(const ldpc_code *c, const ResidentShape &sh, const f
     a.v16 = reinterpret_cast<const uint4 *>(p.tab + p.off[vt + 2]);
     a.n_cg = p.n_cg;
     a.n_vg = p.n_vg;
+    a.n_v1 = p.n_v1;
     a.n_v3 = p.n_v3;
     a.n_v8 = p.n_v8;
     a.n_v16 = p.n_v16;

@@ -25,7 +25,8 @@ namespace ldpc {
 // variables, 32 for messages, a table per message size): a shared-memory access
 // then takes no address arithmetic but the row's unpacking. A missing entry of a check is
 // kResidentPad; a missing edge of a variable is the slot past the last one,
-// whose message is always -0. The checks of degree above 32 and the variables
+// whose message is always -0 (+0 in int8, which has no other zero, so that a sum
+// with at least one message is the same). The checks of degree above 32 and the variables
 // of degree above kWideVarDegree follow, each worked on by a warp.
 constexpr uint16_t kResidentPad = 0xFFFF;
 
@@ -33,7 +34,7 @@ struct ResidentPlan {
     bool ok = false;
     int32_t slots = 0;   // message slots (padding included, the -0 slot not)
     int32_t dclass = 0;  // inputs the check rows have room for: 4, 6 or 8 (rows of 8), 12, 18 (20) or 32
-    int32_t n_cg = 0, n_vg = 0, n_v3 = 0, n_v8 = 0, n_v16 = 0;  // groups; of them with variables of degree above 2, 4, 8
+    int32_t n_cg = 0, n_vg = 0, n_v1 = 0, n_v3 = 0, n_v8 = 0, n_v16 = 0;  // groups; of them with variables of degree above 0, 2, 4, 8
     int32_t n_wc = 0, n_wv = 0;
     size_t off[15] = {0};          // byte offsets in tab of the tables below, in order
     unsigned char *tab = nullptr;  // device
@@ -60,7 +61,7 @@ struct ResidentArgs {
     const uint16_t *var;         // [n_vg * 32 + n_wv] variable of an internal index
     const int4 *wide;            // n_wc checks (first slot, degree, first entry in list), n_wv variables (first entry, degree, internal index)
     const uint16_t *list;        // entries of the wide nodes
-    int32_t n_cg, n_vg, n_v3, n_v8, n_v16, n_wc, n_wv;
+    int32_t n_cg, n_vg, n_v1, n_v3, n_v8, n_v16, n_wc, n_wv;
     int32_t n, F, f0, slots;  // frames f0 + blockIdx.x
     int32_t max_iter, early;
     int32_t lam_shared;  // channel LLRs kept in shared memory (else re-read from llr)

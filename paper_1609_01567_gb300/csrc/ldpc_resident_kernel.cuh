@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
         gr.r = r + (int)(cw & 0xFFFFu) * 32 + lane;
     };
     auto fetch_var = [&](int g) {
-        if (g < a.n_vg) vv = __ldg(a.v4 + g * 32 + lane);
+        if (g < a.n_v1) vv = __ldg(a.v4 + g * 32 + lane);
     };
     if constexpr (kAhead) fetch_check(warp);
 
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(max_threads<DC, RULE>(), 1) k_resident(const _
         sum_edges(std::integral_constant<int, 16>{}, a.n_v16);  // groups are in falling order of degree
         sum_edges(std::integral_constant<int, 8>{}, a.n_v8);
         sum_edges(std::integral_constant<int, 4>{}, a.n_v3);
-        sum_edges(std::integral_constant<int, 2>{}, a.n_vg);
+        sum_edges(std::integral_constant<int, 2>{}, a.n_v1);  // those without a check keep what they have
         // variables of degree above kWideVarDegree: eight partial sums (lane u
         // over edges u, u + 8, ...) added to lambda in order
         for (int g = warps - 1 - warp; g < a.n_wv; g += warps) {

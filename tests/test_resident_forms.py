@@ -173,3 +173,22 @@ def test_nan_inputs(ldpc, degrees, frames):  # noqa: F811
                     assert torch.equal(torch.nan_to_num(got[k].float(), 123.0), torch.nan_to_num(ref[k].float(), 123.0)), (
                         msg, rule, max_iter, k)
                 assert torch.equal(got["post"].isnan(), ref["post"].isnan())
+
+
+@pytest.mark.parametrize("msg", ["f32", "f16", "bf16", "i8"])
+def test_variables_without_a_check(ldpc, msg):  # noqa: F811
+    """Their posteriors are their channel values, -0 included, in every format."""
+    m, n = 40, 600
+    rows, cols = random_code(m, n, [3, 6], seed=1)
+    free = np.setdiff1d(np.arange(n), cols)
+    assert free.size > 300
+    h = ldpc.ldpc_code_create(m, n, rows, cols)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    llr = torch.randn((40, n), generator=gen, device="cuda") * 4.0
+    llr[:, ::3] = -0.0
+    got, ref = decodes(ldpc, h, llr, 5, early_exit=False, msg_dtype=msg)
+    for k in ref:
+        a, b = (x.view(torch.int32) if x.dtype == torch.float32 else x for x in (got[k], ref[k]))  # -0 is not +0
+        assert torch.equal(a, b), k
+    at = torch.from_numpy(free).cuda()
+    assert torch.equal(got["post"][:, at].view(torch.int32), llr[:, at].view(torch.int32))
