@@ -539,8 +539,11 @@ cudaError_t launch_frames(const ResidentArgs &a, int32_t frames, const ResidentS
         ready[dev & 63].store(true, std::memory_order_release);
     }
     const unsigned threads = (unsigned)std::min(sh.threads, max_threads<DC, RULE>());
-    k_resident<M, DC, RULE, ZN><<<(unsigned)frames, threads, sh.smem, s>>>(a);
-    return cudaGetLastError();
+    // the launch's own status: cudaGetLastError would also report what an earlier,
+    // refused call left (a decode that was refused inside a capture)
+    void *args[] = {const_cast<ResidentArgs *>(&a)};
+    return cudaLaunchKernel(reinterpret_cast<const void *>(k_resident<M, DC, RULE, ZN>), dim3((unsigned)frames),
+                            dim3(threads), args, sh.smem, s);
 }
 
 template <typename M, int DC, int RULE>

@@ -1,5 +1,9 @@
 """Forms of the resident decode that depend on a code's mixture of degrees,
 compared bit for bit with the pass kernels (a profiled decode runs those)."""
+import subprocess
+import sys
+from pathlib import Path
+
 import numpy as np
 import pytest
 
@@ -8,6 +12,8 @@ from tests.test_resident import decodes, ldpc, random_code  # noqa: F401  (ldpc 
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+ROOT = Path(__file__).resolve().parent.parent
 
 
 # Checks on both sides of degree 16, whose sign rule for an input of exactly +0
@@ -192,3 +198,28 @@ def test_variables_without_a_check(ldpc, msg):  # noqa: F811
         assert torch.equal(a, b), k
     at = torch.from_numpy(free).cuda()
     assert torch.equal(got["post"][:, at].view(torch.int32), llr[:, at].view(torch.int32))
+
+
+REFUSED_IN_A_CAPTURE = """
+import torch
+from paper_1609_01567_gb300 import inputs, ldpc
+code = inputs.small_code_n1008()
+h = ldpc.code_from_inputs(code)
+llr = torch.full((8, code.n), -3.0, device="cuda")
+out = ldpc.ldpc_decode(h, llr, 5)
+torch.cuda.synchronize()
+refused = False
+try:
+    with torch.cuda.graph(torch.cuda.CUDAGraph()):
+        ldpc.ldpc_decode(h, llr, 5, out=out)  # waits for the decode before it, which the capture does not hold
+except Exception:
+    refused = True
+again = ldpc.ldpc_decode(h, llr, 5)
+torch.cuda.synchronize()
+assert refused and not again["bits"].any() and again["ok"].all()
+"""
+
+
+def test_decode_after_one_that_a_capture_refused(ldpc):  # noqa: F811
+    r = subprocess.run([sys.executable, "-c", REFUSED_IN_A_CAPTURE], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
