@@ -514,18 +514,25 @@ cudaError_t encoder_rows_create(ldpc_code *c) {
     try {
         std::vector<int2> groups;
         std::vector<uint32_t> rows;
+        rows.reserve((size_t)c->E);
         for (int32_t i0 = 0; i0 < c->m; i0 += 32) {
             const int32_t i1 = std::min(c->m, i0 + 32);
-            std::vector<std::vector<uint32_t>> in(32);
-            size_t width = 0;
+            int32_t in[32] = {0}, width = 0;  // information columns of a check
             for (int32_t i = i0; i < i1; ++i) {
-                for (int32_t e = c->row_ptr[i]; e < c->row_ptr[i + 1]; ++e)
-                    if ((uint32_t)c->col_idx[e] < k) in[i - i0].push_back((uint32_t)c->col_idx[e]);
-                width = std::max(width, in[i - i0].size());
+                for (int32_t e = c->row_ptr[i]; e < c->row_ptr[i + 1]; ++e) in[i - i0] += (uint32_t)c->col_idx[e] < k;
+                width = std::max(width, in[i - i0]);
             }
-            groups.push_back(make_int2((int)rows.size(), (int)width));
-            for (size_t e = 0; e < width; ++e)
-                for (int l = 0; l < 32; ++l) rows.push_back(e < in[l].size() ? in[l][e] : k);
+            const size_t first = rows.size();
+            groups.push_back(make_int2((int)first, width));
+            rows.resize(first + 32 * (size_t)width, k);
+            for (int32_t i = i0; i < i1; ++i) {
+                uint32_t *to = rows.data() + first + (i - i0);
+                for (int32_t e = c->row_ptr[i]; e < c->row_ptr[i + 1]; ++e) {
+                    if ((uint32_t)c->col_idx[e] >= k) continue;
+                    *to = (uint32_t)c->col_idx[e];
+                    to += 32;
+                }
+            }
             if (rows.size() > 4 * (size_t)c->E + 4096) return cudaSuccess;
         }
         cudaError_t e = cudaMalloc(&c->ira_groups, sizeof(int2) * groups.size());

@@ -15,12 +15,21 @@ namespace ldpc {
 static std::vector<std::vector<int32_t>> degree_groups(std::vector<int32_t> ids, const std::vector<int32_t> &ptr,
                                                        std::initializer_list<int32_t> borders) {
     auto deg = [&](int32_t i) { return ptr[i + 1] - ptr[i]; };
-    std::stable_sort(ids.begin(), ids.end(), [&](int32_t a, int32_t b) { return deg(a) > deg(b); });
+    int32_t top = 0;
+    for (int32_t id : ids) top = std::max(top, deg(id));
+    std::vector<int32_t> at((size_t)top + 2, 0), sorted(ids.size());  // counting sort: creating a code waits for this
+    for (int32_t id : ids) at[top - deg(id) + 1] += 1;
+    for (int32_t d = 0; d <= top; ++d) at[d + 1] += at[d];
+    for (int32_t id : ids) sorted[at[top - deg(id)]++] = id;
+    ids.swap(sorted);
     std::vector<std::vector<int32_t>> groups;
     for (int32_t id : ids) {
         bool cut = groups.empty() || groups.back().size() == 32;
         for (int32_t b : borders) cut = cut || (deg(groups.back()[0]) > b && deg(id) <= b);
-        if (cut) groups.emplace_back();
+        if (cut) {
+            groups.emplace_back();
+            groups.back().reserve(32);
+        }
         groups.back().push_back(id);
     }
     return groups;
@@ -86,6 +95,7 @@ static cudaError_t make_plan(const ldpc_code *c, ResidentPlan *p) {
     // 16-bit slots, and one frame's smallest messages must fit
     if (slots >= kResidentPad || (size_t)c->n * 4 + (size_t)slots + 64 > (size_t)kResidentSmem) return cudaSuccess;
     std::vector<uint32_t> v4, v8, v16;
+    v4.reserve(vg.size() * 128);
     for (const auto &g : vg) {
         const int32_t d0 = degree(c->col_ptr, g[0]);
         p->n_v1 += d0 > 0 ? 1 : 0;
