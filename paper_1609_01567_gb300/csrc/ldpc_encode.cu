@@ -320,6 +320,7 @@ cudaError_t launch_encode_ira(const uint8_t *info, const int2 *groups, const uin
 // columns of eight words: lane q takes four bytes of each of a word's 32
 // frames, from the one or two aligned words that hold them (rows of k bytes
 // start anywhere), and the tile leaves as 32-byte runs.
+template <bool kEnds>
 __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ info, int32_t F, int32_t k, int32_t Gp,
                                                     uint32_t *__restrict__ U, uint32_t *__restrict__ P,
                                                     int64_t p_words) {
@@ -332,18 +333,25 @@ __global__ void __launch_bounds__(256) k_dense_pack(const uint8_t *__restrict__ 
     const int32_t g = blockIdx.y * 8 + warp;
     const int need = min(4, k - j);  // columns of this lane; more bytes than that go nowhere
     uint32_t w[4] = {0u, 0u, 0u, 0u};
-    // The words that hold info's first and last byte reach past its ends where
-    // these are unaligned: put together from their bytes inside it. (Byte loads of
-    // all columns at the ends instead: up to 4 us longer.)
-    const uintptr_t lo = reinterpret_cast<uintptr_t>(info), hi = lo + (size_t)F * k;
-    const uintptr_t first = lo & 3 ? lo & ~(uintptr_t)3 : 0, last = hi & 3 ? hi & ~(uintptr_t)3 : 0;
+    // kEnds: info's first or last byte is unaligned, so that the word that holds it
+    // reaches past the buffer: put together from its bytes inside. (For all calls:
+    // n = 8192, 1000 frames 40.7 us instead of 38.9; byte loads of all columns at the
+    // ends: up to 4 us longer.)
+    uintptr_t first = 0, last = 0;
     uint32_t head = 0, tail = 0;
+    if constexpr (kEnds) {
+        const uintptr_t lo = reinterpret_cast<uintptr_t>(info), hi = lo + (size_t)F * k;
+        first = lo & 3 ? lo & ~(uintptr_t)3 : 0;
+        last = hi & 3 ? hi & ~(uintptr_t)3 : 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (first && first + i >= lo && first + i < hi) head |= (uint32_t)*reinterpret_cast<const uint8_t *>(first + i) << (8 * i);
-        if (last && last + i >= lo && last + i < hi) tail |= (uint32_t)*reinterpret_cast<const uint8_t *>(last + i) << (8 * i);
+        for (int i = 0; i < 4; ++i) {
+            const uintptr_t h = first + i, t = last + i;
+            if (first && h >= lo && h < hi) head |= (uint32_t)*reinterpret_cast<const uint8_t *>(h) << (8 * i);
+            if (last && t >= lo && t < hi) tail |= (uint32_t)*reinterpret_cast<const uint8_t *>(t) << (8 * i);
+        }
     }
     auto word = [&](uintptr_t a) {
+        if (!kEnds) return *reinterpret_cast<const uint32_t *>(a);
         uint32_t x = a == first ? head : tail;
         if (a != first && a != last) x = *reinterpret_cast<const uint32_t *>(a);
         return x;
@@ -756,7 +764,8 @@ extern "C" int ldpc_encode(ldpc_code_t *c, const uint8_t *info, int32_t n_frames
             const uint8_t *in = info + (size_t)f0 * k;
             uint8_t *out = codeword + (size_t)f0 * n;
             const dim3 pack((unsigned)std::max((k + 127) / 128, 1), (unsigned)(Gp / 8));
-            k_dense_pack<<<pack, 256, 0, s>>>(in, F, k, Gp, U, P, (int64_t)r * Gp);
+            const bool ends = ((reinterpret_cast<uintptr_t>(in) | (uintptr_t)((int64_t)F * k)) & 3) != 0;
+            (ends ? k_dense_pack<true> : k_dense_pack<false>)<<<pack, 256, 0, s>>>(in, F, k, Gp, U, P, (int64_t)r * Gp);
             if (r > 0 && k > 0) {
                 const dim3 grid((unsigned)blocks, (unsigned)((kw + slice - 1) / slice), (unsigned)(Gp / 32));
                 k_dense_parity<<<grid, 256, 0, s>>>(c->enc_R, r, k, kw, slice, U, Gp, P);
