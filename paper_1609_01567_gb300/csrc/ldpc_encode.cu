@@ -125,7 +125,7 @@ __global__ void k_write_codeword(const uint8_t *__restrict__ info, const uint32_
 // the lanes' entries next to each other, with a running xor by shuffles; after
 // one barrier for the warps' totals it writes its range as bytes of the eight
 // rows, W bytes a store. Bound by the bytes read and written once and by the
-// latency of the table rows between them: n = 64800, 1024 frames 259 -> 36 us
+// latency of the table rows between them: n = 64800, 1024 frames 259 -> 36-39 us
 // against the four kernels of the general path, whose write kernel divides a
 // 64-bit index for every codeword byte (100 MB at the copy rate: 15 us). Rows
 // read through row_ptr and col_idx instead of the padded table: 54 us, every

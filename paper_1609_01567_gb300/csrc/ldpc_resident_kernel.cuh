@@ -12,11 +12,12 @@
 // through HBM or L2 three times a pass, launch at least two kernels a pass up to
 // max_iter, and keep a group of 64-128 frames running until its last one stops;
 // here a frame costs its own iterations. Measured (pass kernels -> this one,
-// early exit unless said): n = 1008, one frame 149 -> 17 us, 1000 frames 576 ->
-// 160 us; n = 2048 (4, 8)-regular, 10,000 frames with channel noise and error
-// count 5.74 -> 1.90 ms; n = 8192, 700 frames 916 -> 341 us; n = 8192 with a
-// degree-96 check, bfloat16, 256 frames, 10 fixed iterations 272 -> 176 us; n =
-// 16200 min-sum, 301 frames 1.40 -> 0.83 ms. Two frames a CTA in packed FP32
+// early exit unless said): n = 1008, one frame 149-180 -> 17-25 us with the call,
+// 1000 frames 576 -> 162 us; n = 2048 (4, 8)-regular, 10,000 frames with channel
+// noise and error count 5.74 -> 1.90 ms; n = 8192, 700 frames 916 -> 341 us; n =
+// 8192 with a degree-96 check, bfloat16, 256 frames, 10 fixed iterations 271 -> 173
+// us; n = 16200 min-sum, 301 frames 1.41 -> 0.83-0.89 ms. These are frames that stop;
+// resident_shape weighs frames that do not. Two frames a CTA in packed FP32
 // pairs were slower for all but fixed iterations (n = 8192, 700 frames: 916 us):
 // both run to the slower one's end.
 #pragma once
